@@ -190,9 +190,11 @@ __device__ __forceinline__ int floor_div_q(int a, int b) {
 // Window geometry of one motion tile of one frame for Q = 2 x (output px per raw px
 // numerator): {floor(Q vx), floor(Q vy)} exactly and the fractions {Q vx - F, Q vy - F}
 // (Sec. 5.1: the window centre and the kernel's sampling point).  The base frame's entry
-// is zero: its motion is zero by definition.  i runs over n x tiles.
+// is zero: its motion is zero by definition.  i runs over n x tiles.  split: each integer F
+// comes as (F div 2Q) << 6 | F mod 2Q (a half-res cell and a phase, 2Q <= 32); motion that
+// takes every window far outside any frame is clamped to 2^26 / Q px.
 __device__ __forceinline__ void geo_entry(const float2 *__restrict__ motion, int n, int ntl, int ref, int Q,
-                                          int4 *__restrict__ geo, int i) {
+                                          int4 *__restrict__ geo, int i, bool split) {
     if (i >= n * ntl) return;
     int4 e = make_int4(0, 0, 0, 0);
     if (i / ntl != ref) {
@@ -200,6 +202,15 @@ __device__ __forceinline__ void geo_entry(const float2 *__restrict__ motion, int
         const int FX = floor_mul(Q, mv.x), FY = floor_mul(Q, mv.y);
         const float fQ = (float)Q;
         e = make_int4(FX, FY, __float_as_int(fmaf(fQ, mv.x, -(float)FX)), __float_as_int(fmaf(fQ, mv.y, -(float)FY)));
+        if (split) {
+            constexpr int kLim = 1 << 26;
+            const int cx = clampi(FX, -kLim, kLim), cy = clampi(FY, -kLim, kLim);
+            const int qx = floor_div(cx, 2 * Q), qy = floor_div(cy, 2 * Q);
+            e.x = qx * 64 + (cx - qx * 2 * Q);
+            e.y = qy * 64 + (cy - qy * 2 * Q);
+            if (cx != FX) e.z = 0;
+            if (cy != FY) e.w = 0;
+        }
     }
     HMFSR_ST(geo + i, e);
 }

@@ -19,7 +19,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "accumulate.cuh"
+#include "accumulate_region.cuh"
 
 namespace hmfsr {
 namespace {
@@ -101,6 +101,12 @@ __device__ __host__ inline int stage_k(int s) {
     }
 }
 
+template <int SN, int SD>
+__device__ __host__ inline int region_subs(const Geom &g) {
+    return stage::region_count<SN, SD>(g.w) * stage::region_count<SN, SD>(g.h) *
+           div_up(stage::region_items<SN, SD, 1>(), kBatchThreads);
+}
+
 // number of 128-thread sub-items of stage s of one burst (mw x mh: accumulation item shape)
 __device__ __host__ inline int stage_subitems(const BatchBurst &b, int s, int mw, int mh) {
     const Geom &g = b.g;
@@ -119,9 +125,13 @@ __device__ __host__ inline int stage_subitems(const BatchBurst &b, int s, int mw
         case S_LK: return div_up(b.L.lty[0] * b.L.ltx[0], kLkTiles) * g.n;
         case S_STRENGTH: return div_up(g.n * g.ty * g.tx, kBatchThreads);
         case S_ROB: return div_up(g.wh, 4 * stage::kRobOut) * div_up(g.hh, stage::kRobStrip) * (g.n - 1);
-        case S_MERGE:  // scale 1: blocks of 32 x 16 pixels in 2 x 2 quads (merge_quad1)
-            return b.snum == b.sden ? div_up(b.wo, stage::kQuadW) * div_up(b.ho, 8 * stage::kQuadNY)
-                                    : div_up(b.wo, mw) * div_up(b.ho, mh);
+        case S_MERGE:  // scales 1, 3/2, 2: a region's items, 128 at a time (merge_region)
+            switch (stage::region_kind(g.tile, b.snum, b.sden)) {
+                case 1: return region_subs<1, 1>(g);
+                case 2: return region_subs<3, 2>(g);
+                case 3: return region_subs<2, 1>(g);
+                default: return div_up(b.wo, mw) * div_up(b.ho, mh);
+            }
         default: return 0;
     }
 }
@@ -143,14 +153,25 @@ __device__ __forceinline__ void run_ssd(const BatchBurst &b, int l, int tile, in
                            top ? 0 : L.lty[l + 1], top ? 0 : L.ltx[l + 1], fsh, b.g.ref, L.vec[l], tile, f);
 }
 
+// shared memory of the accumulation: the largest scale's
+union MergeSmem {
+    stage::RegionSmem<2> s2;
+    stage::RegionSmem<3> s3;
+    stage::RegionSmem<4> s4;
+};
+
 template <int SN, int SD>
-__device__ __forceinline__ void run_merge(const BatchBurst &b, int X, int Y) {
-    stage::merge_px<false, SN, SD>(b.burst, b.P.geo, b.g, b.P.kern, b.P.rhat,
-                                   b.snum, b.sden, b.ho, b.wo, b.rgb, nullptr, X, Y);
+__device__ __forceinline__ void run_region(const BatchBurst &b, void *smem, int k, int tid) {
+    constexpr int nz = (stage::region_items<SN, SD, 1>() + kBatchThreads - 1) / kBatchThreads;
+    const int nx = stage::region_count<SN, SD>(b.g.w), z = k % nz, r = k / nz;
+    __syncthreads();  // the previous region's last frame has been read
+    stage::merge_region<false, SN, SD, kBatchThreads, 1>(  // one x phase per thread, for the smaller register builds
+        *static_cast<stage::RegionSmem<stage::RegionScale<SN, SD>::S> *>(smem), b.burst, b.P.geo, b.g, b.P.kern, b.P.rhat,
+        b.ho, b.wo, b.rgb, nullptr, r % nx, r / nx, z * kBatchThreads, tid);
 }
 
 // one sub-item of one stage of burst b, by all 128 threads of the block
-__device__ __forceinline__ void run_sub(const BatchBurst &b, int s, int k, int tid, int mw, int mh) {
+__device__ __forceinline__ void run_sub(const BatchBurst &b, int s, int k, int tid, int mw, int mh, void *smem) {
     const Geom &g = b.g;
     const float2 *mv = reinterpret_cast<const float2 *>(b.motion);
     switch (s) {
@@ -197,7 +218,8 @@ __device__ __forceinline__ void run_sub(const BatchBurst &b, int s, int k, int t
         }
         case S_STRENGTH:
             stage::strength(mv, g.n, g.ty, g.tx, b.c.m_th, b.c.s1, b.c.s2, b.P.s_tile, k * kBatchThreads + tid);
-            stage::geo_entry(mv, g.n, g.ty * g.tx, g.ref, 2 * b.snum, b.P.geo, k * kBatchThreads + tid);
+            stage::geo_entry(mv, g.n, g.ty * g.tx, g.ref, stage::geo_q(g.tile, b.snum, b.sden), b.P.geo,
+                             k * kBatchThreads + tid, stage::region_kind(g.tile, b.snum, b.sden) != 0);
             break;
         case S_ROB: {
             const int nx = div_up(g.wh, 4 * stage::kRobOut), ny = div_up(g.hh, stage::kRobStrip);
@@ -208,23 +230,16 @@ __device__ __forceinline__ void run_sub(const BatchBurst &b, int s, int k, int t
             break;
         }
         case S_MERGE: {
-            if (b.snum == b.sden) {
-                // the per-burst kernel's layout: 4 warps of 8 x 4 threads of 2 x kQuadNY pixels
-                constexpr int NY = stage::kQuadNY;
-                const int nx = div_up(b.wo, stage::kQuadW), by = k / nx, bx = k - by * nx;
-                const int w = tid >> 5, lane = tid & 31;
-                const int qx = (w & 1) * 8 + (lane & 7), qy = (w >> 1) * 4 + (lane >> 3);
-                stage::merge_quad1<false, NY>(b.burst, b.P.geo, b.g, b.P.kern, b.P.rhat, b.rgb, nullptr,
-                                              bx * stage::kQuadW + 2 * qx, by * 8 * NY + NY * qy);
-                break;
+            switch (stage::region_kind(g.tile, b.snum, b.sden)) {
+                case 1: run_region<1, 1>(b, smem, k, tid); break;
+                case 2: run_region<3, 2>(b, smem, k, tid); break;
+                case 3: run_region<2, 1>(b, smem, k, tid); break;
+                default: {
+                    const int nx = div_up(b.wo, mw), by = k / nx, bx = k - by * nx;
+                    stage::merge_px<false, 0, 0>(b.burst, b.P.geo, b.g, b.P.kern, b.P.rhat, b.snum, b.sden, b.ho, b.wo,
+                                                 b.rgb, nullptr, bx * mw + tid % mw, by * mh + tid / mw);
+                }
             }
-            const int nx = div_up(b.wo, mw);
-            const int by = k / nx, bx = k - by * nx;
-            const int X = bx * mw + tid % mw, Y = by * mh + tid / mw;
-            if (b.snum == 1 && b.sden == 1) run_merge<1, 1>(b, X, Y);
-            else if (b.snum == 3 && b.sden == 2) run_merge<3, 2>(b, X, Y);
-            else if (b.snum == 2 && b.sden == 1) run_merge<2, 1>(b, X, Y);
-            else run_merge<0, 0>(b, X, Y);
             break;
         }
         default: break;
@@ -232,12 +247,12 @@ __device__ __forceinline__ void run_sub(const BatchBurst &b, int s, int k, int t
 }
 
 // one queue item: stage_k(s) consecutive sub-items
-__device__ __forceinline__ void run_item(const BatchBurst &b, int s, int k, int tid, int mw, int mh) {
+__device__ __forceinline__ void run_item(const BatchBurst &b, int s, int k, int tid, int mw, int mh, void *smem) {
     const int K = stage_k(s), nsub = stage_subitems(b, s, mw, mh);
     for (int j = 0; j < K; ++j) {
         const int sub = k * K + j;
         if (sub >= nsub) break;
-        run_sub(b, s, sub, tid, mw, mh);
+        run_sub(b, s, sub, tid, mw, mh, smem);
     }
 }
 
@@ -260,6 +275,7 @@ __global__ void __launch_bounds__(kBatchThreads, MINB)
     k_batch(const BatchBurst *__restrict__ bursts, const Segment *__restrict__ segs, int nseg, int total,
             int *ctrl, int *done, const int *__restrict__ totals, int mw, int mh, int spin_limit,
             unsigned long long *prof) {
+    __shared__ MergeSmem s_merge;
     __shared__ int s_item, s_next, s_ok, s_seg;
     __shared__ long long s_t1;
     __shared__ unsigned int s_ready[kMaxCachedBursts];  // per burst: bit s set once stage s is complete
@@ -315,7 +331,7 @@ __global__ void __launch_bounds__(kBatchThreads, MINB)
         if (item >= total || !s_ok) break;
         const Segment sg = segs[s_seg];
         const int b = sg.burst, s = sg.stage, k = item - sg.first;
-        run_item(bursts[b], s, k, tid, mw, mh);
+        run_item(bursts[b], s, k, tid, mw, mh, &s_merge);
         __syncthreads();
         if (tid == 0) {
             add_release(&done[b * S_COUNT + s], 1);
@@ -346,7 +362,9 @@ struct hmfsr_batch_plan_t {
     size_t table_off = 0, seg_off = 0, tot_off = 0, done_off = 0, ctrl_off = 0, prof_off = 0, ws_bytes = 0;
     int profile = 0;  // the persistent kernel sums per-stage cycles (hmfsr_batch_set_profile)
     int mw = 32, mh = 4, ctas_per_sm = 0;  // accumulation item shape, blocks per SM (0: all that fit)
-    int regs_variant = 1;                  // kernel build: 0 = 128, 1 = 80, 2 = 64 registers per thread
+    // kernel build: 0 = 128, 1 = 80, 2 = 64 registers per thread.  128 is the fastest untuned: the
+    // region accumulation spills below (six bursts of 0.5-3 MP: 3.81, 5.05, 5.92 ms)
+    int regs_variant = 0;
     int mode = 0;                          // 0: one persistent kernel; k > 0: graph of per-burst kernels on k streams
     int order = 0;                         // queue: 0 = stage-major, 1 = burst-major
     int spin_limit = 1 << 22;

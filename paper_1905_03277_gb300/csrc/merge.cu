@@ -4,7 +4,7 @@
 // live in stages.cuh, shared with the batched persistent kernel.
 #include <atomic>
 
-#include "accumulate.cuh"
+#include "accumulate_region.cuh"
 
 namespace hmfsr {
 namespace {
@@ -44,8 +44,9 @@ __global__ void k_hf_flag(const uint16_t *__restrict__ burst, const uint2 *__res
     stage::hf_flag_px(burst, s1, g, kappa, flag, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y);
 }
 
-__global__ void k_geo(const float2 *__restrict__ motion, int n, int ntl, int ref, int Q, int4 *__restrict__ geo) {
-    stage::geo_entry(motion, n, ntl, ref, Q, geo, blockIdx.x * blockDim.x + threadIdx.x);
+__global__ void k_geo(const float2 *__restrict__ motion, int n, int ntl, int ref, int Q, int4 *__restrict__ geo,
+                      bool split) {
+    stage::geo_entry(motion, n, ntl, ref, Q, geo, blockIdx.x * blockDim.x + threadIdx.x, split);
 }
 
 template <bool kDen, int SN, int SD>
@@ -101,36 +102,70 @@ __global__ void __launch_bounds__(128, (NY == 2 ? 4 : 5)) k_merge_q1_chunk(const
                                        blockIdx.x * stage::kQuadW + 2 * qx, blockIdx.y * 8 * NY + NY * qy, io);
 }
 
-template <bool kDen>
-static void launch_k_merge_chunk(dim3 grid, cudaStream_t s, const uint16_t *burst, const int4 *mv, const Geom &g,
-                                 const MergePlanes &P, int snum, int sden, int ho, int wo, float *rgb, float *den,
-                                 const stage::ChunkIO &io) {
-    const dim3 block(kMergeW, kMergeH);
-    if (snum == sden)
-        k_merge_q1_chunk<kDen, stage::kQuadNY>
-            <<<dim3(div_up(wo, stage::kQuadW), div_up(ho, 8 * stage::kQuadNY)), 128, 0, s>>>(burst, mv, g, P.kern,
-                                                                                             P.rhat, rgb, den, io);
-    else if (snum == 3 && sden == 2)
-        k_merge_chunk<kDen, 3, 2><<<grid, block, 0, s>>>(burst, mv, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den, io);
-    else if (snum == 2 && sden == 1)
-        k_merge_chunk<kDen, 2, 1><<<grid, block, 0, s>>>(burst, mv, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den, io);
-    else
-        k_merge_chunk<kDen, 0, 0><<<grid, block, 0, s>>>(burst, mv, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den, io);
+// A region's output pixels (stage::merge_region): threads and blocks per SM by scale.  Measured
+// on the 12-MP bursts (accumulation call): 1x, 128 threads: 5 blocks per SM 930 us, 6 (spills)
+// 965, 4 1006; 1.5x, 288 threads: 3 blocks 1921 us, 2 2125; 2x, 256 threads, two x phases each:
+// 2 blocks 5315 us (128 threads x 4 5605; one phase each, 256 x 3, 6076).
+template <int SN, int SD>
+struct RegionShape;
+template <> struct RegionShape<1, 1> { static constexpr int kThreads = 128, kBlocks = 5, kNpx = 1; };
+template <> struct RegionShape<3, 2> { static constexpr int kThreads = 288, kBlocks = 3, kNpx = 1; };
+template <> struct RegionShape<2, 1> { static constexpr int kThreads = 256, kBlocks = 2, kNpx = 2; };
+
+template <bool kDen, int SN, int SD, bool kChunk>
+__global__ void __launch_bounds__(RegionShape<SN, SD>::kThreads, RegionShape<SN, SD>::kBlocks)
+    k_merge_region(const uint16_t *__restrict__ burst, const int4 *__restrict__ geo, Geom g,
+                   const float4 *__restrict__ kern, const float *__restrict__ rhat_planes, int ho, int wo,
+                   float *__restrict__ rgb, float *__restrict__ den_out, stage::ChunkIO io) {
+    constexpr int NT = RegionShape<SN, SD>::kThreads, NPX = RegionShape<SN, SD>::kNpx;
+    static_assert(stage::region_items<SN, SD, NPX>() == NT, "one block per region");
+    __shared__ stage::RegionSmem<stage::RegionScale<SN, SD>::S> sm;
+    stage::merge_region<kDen, SN, SD, NT, NPX, kChunk>(sm, burst, geo, g, kern, rhat_planes, ho, wo, rgb, den_out,
+                                                  blockIdx.x, blockIdx.y, 0, threadIdx.x, io);
 }
 
-template <bool kDen>
-static void launch_k_merge(dim3 grid, cudaStream_t s, const uint16_t *burst, const int4 *mv, const Geom &g,
-                           const MergePlanes &P, int snum, int sden, int ho, int wo, float *rgb, float *den) {
-    const dim3 block(kMergeW, kMergeH);
-    if (snum == sden)
-        k_merge_q1<kDen, stage::kQuadNY><<<dim3(div_up(wo, stage::kQuadW), div_up(ho, 8 * stage::kQuadNY)), 128, 0, s>>>(
-            burst, mv, g, P.kern, P.rhat, rgb, den);
-    else if (snum == 3 && sden == 2)
-        k_merge<kDen, 3, 2><<<grid, block, 0, s>>>(burst, mv, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den);
-    else if (snum == 2 && sden == 1)
-        k_merge<kDen, 2, 1><<<grid, block, 0, s>>>(burst, mv, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den);
-    else
-        k_merge<kDen, 0, 0><<<grid, block, 0, s>>>(burst, mv, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den);
+template <bool kDen, int SN, int SD, bool kChunk>
+static void launch_region(cudaStream_t s, const uint16_t *burst, const Geom &g, const MergePlanes &P, int ho, int wo,
+                          float *rgb, float *den, const stage::ChunkIO &io) {
+    k_merge_region<kDen, SN, SD, kChunk>
+        <<<dim3(stage::region_count<SN, SD>(g.w), stage::region_count<SN, SD>(g.h)), RegionShape<SN, SD>::kThreads, 0, s>>>(
+            burst, P.geo, g, P.kern, P.rhat, ho, wo, rgb, den, io);
+}
+
+// the accumulation's kernel for a tile size and scale (geometry in P.geo, geo_q)
+template <bool kDen, bool kChunk>
+static void launch_k_merge(cudaStream_t s, const uint16_t *burst, const Geom &g, const MergePlanes &P, int snum, int sden,
+                           int ho, int wo, float *rgb, float *den, const stage::ChunkIO &io) {
+    switch (stage::region_kind(g.tile, snum, sden)) {
+        case 1: return launch_region<kDen, 1, 1, kChunk>(s, burst, g, P, ho, wo, rgb, den, io);
+        case 2: return launch_region<kDen, 3, 2, kChunk>(s, burst, g, P, ho, wo, rgb, den, io);
+        case 3: return launch_region<kDen, 2, 1, kChunk>(s, burst, g, P, ho, wo, rgb, den, io);
+        default: break;
+    }
+    const dim3 block(kMergeW, kMergeH), grid(div_up(wo, kMergeW), div_up(ho, kMergeH));
+    if (snum == sden) {
+        const dim3 qgrid(div_up(wo, stage::kQuadW), div_up(ho, 8 * stage::kQuadNY));
+        if constexpr (kChunk)
+            k_merge_q1_chunk<kDen, stage::kQuadNY><<<qgrid, 128, 0, s>>>(burst, P.geo, g, P.kern, P.rhat, rgb, den, io);
+        else
+            k_merge_q1<kDen, stage::kQuadNY><<<qgrid, 128, 0, s>>>(burst, P.geo, g, P.kern, P.rhat, rgb, den);
+        return;
+    }
+    if constexpr (kChunk) {
+        if (snum == 3 && sden == 2)
+            k_merge_chunk<kDen, 3, 2><<<grid, block, 0, s>>>(burst, P.geo, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den, io);
+        else if (snum == 2 && sden == 1)
+            k_merge_chunk<kDen, 2, 1><<<grid, block, 0, s>>>(burst, P.geo, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den, io);
+        else
+            k_merge_chunk<kDen, 0, 0><<<grid, block, 0, s>>>(burst, P.geo, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den, io);
+    } else {
+        if (snum == 3 && sden == 2)
+            k_merge<kDen, 3, 2><<<grid, block, 0, s>>>(burst, P.geo, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den);
+        else if (snum == 2 && sden == 1)
+            k_merge<kDen, 2, 1><<<grid, block, 0, s>>>(burst, P.geo, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den);
+        else
+            k_merge<kDen, 0, 0><<<grid, block, 0, s>>>(burst, P.geo, g, P.kern, P.rhat, snum, sden, ho, wo, rgb, den);
+    }
 }
 
 // --------------------------------------------------------------------------------------
@@ -256,15 +291,15 @@ cudaError_t launch_merge_accum(const uint16_t *burst, const float *motion, const
                                int snum, int sden, float *rgb, float *den, cudaStream_t s) {
     StageRange range("hmfsr merge: accumulation and normalisation");
     CheckedLaunches checked(s);
-    int ho = (int)(((long long)g.h * snum) / sden), wo = (int)(((long long)g.w * snum) / sden);
-    dim3 grid(div_up(wo, kMergeW), div_up(ho, kMergeH));
+    const int ho = (int)(((long long)g.h * snum) / sden), wo = (int)(((long long)g.w * snum) / sden);
     const int ntl = g.ty * g.tx;
-    k_geo<<<div_up(g.n * ntl, 128), 128, 0, s>>>(reinterpret_cast<const float2 *>(motion), g.n, ntl, g.ref, 2 * snum,
-                                                 P.geo);
+    k_geo<<<div_up(g.n * ntl, 128), 128, 0, s>>>(reinterpret_cast<const float2 *>(motion), g.n, ntl, g.ref,
+                                                 stage::geo_q(g.tile, snum, sden), P.geo,
+                                                 stage::region_kind(g.tile, snum, sden) != 0);
     if (den)
-        launch_k_merge<true>(grid, s, burst, P.geo, g, P, snum, sden, ho, wo, rgb, den);
+        launch_k_merge<true, false>(s, burst, g, P, snum, sden, ho, wo, rgb, den, stage::ChunkIO{});
     else
-        launch_k_merge<false>(grid, s, burst, P.geo, g, P, snum, sden, ho, wo, rgb, nullptr);
+        launch_k_merge<false, false>(s, burst, g, P, snum, sden, ho, wo, rgb, nullptr, stage::ChunkIO{});
     return cudaGetLastError();
 }
 
@@ -274,19 +309,19 @@ cudaError_t launch_merge_accum_chunk(const uint16_t *burst, const float *motion,
     StageRange range("hmfsr merge: accumulation of one chunk of frames");
     CheckedLaunches checked(s);
     const int ho = (int)(((long long)g.h * snum) / sden), wo = (int)(((long long)g.w * snum) / sden);
-    const dim3 grid(div_up(wo, kMergeW), div_up(ho, kMergeH));
     const int ntl = g.ty * g.tx;
-    k_geo<<<div_up(g.n * ntl, 128), 128, 0, s>>>(reinterpret_cast<const float2 *>(motion), g.n, ntl, g.ref, 2 * snum,
-                                                 P.geo);
+    k_geo<<<div_up(g.n * ntl, 128), 128, 0, s>>>(reinterpret_cast<const float2 *>(motion), g.n, ntl, g.ref,
+                                                 stage::geo_q(g.tile, snum, sden), P.geo,
+                                                 stage::region_kind(g.tile, snum, sden) != 0);
     stage::ChunkIO io;
     io.state_in = state_in;
     io.state_out = state_out;
     io.skip_base = skip_base ? 1 : 0;
     io.plane = (size_t)ho * wo;
     if (den && !state_out)
-        launch_k_merge_chunk<true>(grid, s, burst, P.geo, g, P, snum, sden, ho, wo, rgb, den, io);
+        launch_k_merge<true, true>(s, burst, g, P, snum, sden, ho, wo, rgb, den, io);
     else
-        launch_k_merge_chunk<false>(grid, s, burst, P.geo, g, P, snum, sden, ho, wo, rgb, nullptr, io);
+        launch_k_merge<false, true>(s, burst, g, P, snum, sden, ho, wo, rgb, nullptr, io);
     return cudaGetLastError();
 }
 
