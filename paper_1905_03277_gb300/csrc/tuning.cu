@@ -7,6 +7,7 @@
 // The mean comes from an exact integer sum of the frame's samples on the GPU
 // (hmfsr_frame_sum); the mapping from SNR to parameters is host arithmetic
 // (hmfsr_snr_tuning).
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "hmfsr_internal.cuh"
@@ -58,7 +59,10 @@ __global__ void __launch_bounds__(kSumThreads) k_frame_sum(const uint16_t *__res
 // Monte-Carlo noise statistics (Sec. 5.2.2: sigma_md and d_md from simulations "for
 // different brightness levels", with sensor clipping)
 // ---------------------------------------------------------------------------------------
-constexpr int kNoiseThreads = 256;
+// a cluster of 8 blocks per brightness level: 1032 blocks of 4 warps, one wave at 7 blocks per
+// SM (one block per level left 23 of 152 SMs idle and 8 warps on each of the others)
+constexpr int kNoiseThreads = 128, kNoiseCluster = 8;
+static_assert(kNoiseTrials % (kNoiseThreads * kNoiseCluster) == 0, "every thread takes the same number of trials");
 
 // Philox-4x32-10 (Salmon et al., SC 2011): ten rounds of two 32x32 -> 64-bit products by
 // fixed multipliers, the halves recombined with the other counter words and the round
@@ -79,86 +83,119 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
 
 // normal j of a trial: 12 uniforms (r + 1/2) 2^-32 from three Philox blocks, summed exactly
 // (Irwin-Hall), minus 6
-__device__ __forceinline__ double noise_normal(int level, int trial, int j) {
-    unsigned long long s = 0;
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        const uint4 o = philox4x32_10(make_uint4((uint32_t)(3 * j + b), (uint32_t)trial, (uint32_t)level, 0u),
-                                      0x19050327u, 0x5EED0001u);
-        s += (unsigned long long)o.x + o.y + o.z + o.w;
-    }
-    return __dadd_rn(__dmul_rn(__dadd_rn((double)s, 6.0), 1.0 / 4294967296.0), -6.0);
+__device__ __forceinline__ uint4 noise_block(int level, int trial, int j, int b) {
+    return philox4x32_10(make_uint4((uint32_t)(3 * j + b), (uint32_t)trial, (uint32_t)level, 0u), 0x19050327u, 0x5EED0001u);
 }
 
 // one raw sample of a constant patch: rounded to a whole DN and clipped to [0, WL], in
 // FP64 with the same operation sequence as a CPU restatement, so every decision agrees
-__device__ __forceinline__ double noise_sample(double x, double sigma, double wl, int level, int trial, int j) {
-    const double v = floor(__dadd_rn(__dadd_rn(x, __dmul_rn(sigma, noise_normal(level, trial, j))), 0.5));
-    return fmin(fmax(v, 0.0), wl);
+__device__ __noinline__ int noise_sample_exact(double x, double sigma, int wl, int level, int trial, int j) {
+    unsigned long long s = 0;
+    for (int b = 0; b < 3; ++b) {
+        const uint4 o = noise_block(level, trial, j, b);
+        s += (unsigned long long)o.x + o.y + o.z + o.w;
+    }
+    const double z = __dadd_rn(__dmul_rn(__dadd_rn((double)s, 6.0), 1.0 / 4294967296.0), -6.0);
+    const double v = floor(__dadd_rn(__dadd_rn(x, __dmul_rn(sigma, z)), 0.5));
+    return (int)fmin(fmax(v, 0.0), (double)wl);
 }
 
-// One block per brightness level; each thread takes every kNoiseThreads-th trial.  A
-// trial draws two independent 3x3 patches of guide pixels (red/blue: one sample; green:
-// the mean of two) and adds {population variance of patch 1, red/blue and green;
-// squared difference of the two patch means, red/blue and green}; the block's FP64 sums
-// become the level's trial means.
-__global__ void __launch_bounds__(kNoiseThreads) k_noise_table(float noise_a, float noise_b, int wl,
-                                                               float4 *__restrict__ table) {
-    __shared__ double red[4][kNoiseThreads];
-    const int level = blockIdx.x;
-    const double x = __ddiv_rn(__dmul_rn((double)level, (double)wl), (double)(kNoiseLevels - 1));
-    const double var = __dadd_rn(__dmul_rn((double)noise_a, x), (double)noise_b);
-    const double sigma = var > 0.0 ? __dsqrt_rn(var) : 0.0;
-    const double dwl = (double)wl;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int t = threadIdx.x; t < kNoiseTrials; t += kNoiseThreads) {
-        double mean[2][2], var1[2];
+// One level's constants.  xi, xh: the brightness x as a whole number plus xh - 1/2 (x is a
+// multiple of 1/128, so both are exact).
+struct NoiseLevel {
+    double x, sigma;
+    float xh, sf, eb;
+    int xi, wl, level;
+};
+
+// The same sample, decided in FP32: floor(xh + sigma z) with z from the uniforms' top 28 bits.
+// Their truncation (12 x 16 x 2^-32 = 4.5e-8), the conversion and the two roundings are below
+// 4e-7 |w| + 2e-7 sigma + 1e-6 of w; only a w closer than that to a whole number (1 sample in
+// 10^4) takes the FP64 sequence, which this GPU issues at 1/64 of the FP32 rate.  All 28.5 M
+// samples in FP64: 863 us; now 1/7 of that or less, bound by the Philox integer products.
+__device__ __forceinline__ int noise_sample(const NoiseLevel &n, int trial, int j) {
+    uint32_t s = 0;
 #pragma unroll
-        for (int ch = 0; ch < 2; ++ch) {
-            double v1[9];
+    for (int b = 0; b < 3; ++b) {
+        const uint4 o = noise_block(n.level, trial, j, b);
+        s += (o.x >> 4) + (o.y >> 4) + (o.z >> 4) + (o.w >> 4);  // 12 x 2^28 < 2^32
+    }
+    const float z = (float)(int)(s - (6u << 28)) * (1.f / 268435456.f);
+    const float w = fmaf(n.sf, z, n.xh), fl = floorf(w), fr = w - fl;
+    const float e = fmaf(4e-7f, fabsf(w), n.eb);
+    if (fabsf(w) < 131072.f && !(fr >= e && fr <= 1.f - e)) return noise_sample_exact(n.x, n.sigma, n.wl, n.level, trial, j);
+    return min(max(n.xi + (int)fminf(fmaxf(fl, -131072.f), 131072.f), 0), n.wl);
+}
+
+// A trial draws two independent 3x3 patches of guide pixels (red/blue: one sample; green: the
+// mean of two).  The statistics of whole numbers are whole numbers over constants, so the level's
+// sums are exact 64-bit integers whatever the order: population variance of patch 1, (9 sum v^2 -
+// (sum v)^2) / 81, red/blue and green (of the doubled green guide, over 4); squared difference of
+// the two patch means, (S1 - S2)^2 / 81, red/blue and green.
+__global__ void __cluster_dims__(kNoiseCluster, 1, 1) __launch_bounds__(kNoiseThreads)
+    k_noise_table(float noise_a, float noise_b, int wl, float4 *__restrict__ table) {
+    namespace cg = cooperative_groups;
+    __shared__ unsigned long long red[kNoiseThreads / 32][4];
+    NoiseLevel n;
+    n.level = blockIdx.x / kNoiseCluster;
+    n.wl = wl;
+    n.x = __ddiv_rn(__dmul_rn((double)n.level, (double)wl), (double)(kNoiseLevels - 1));
+    const double var = __dadd_rn(__dmul_rn((double)noise_a, n.x), (double)noise_b);
+    n.sigma = var > 0.0 ? __dsqrt_rn(var) : 0.0;
+    n.xi = (int)n.x;
+    n.xh = (float)(n.x - (double)n.xi) + 0.5f;
+    n.sf = (float)n.sigma;
+    n.eb = fmaf(2e-7f, n.sf, 1e-6f);
+    unsigned long long acc[4] = {0, 0, 0, 0};
+    constexpr int kPer = kNoiseTrials / (kNoiseThreads * kNoiseCluster);
+    const int t0 = (blockIdx.x % kNoiseCluster) * kNoiseThreads + threadIdx.x;
 #pragma unroll 1
-            for (int q = 0; q < 2; ++q) {
-                double s = 0.0;
+    for (int i = 0; i < kPer; ++i) {
+        const int t = t0 + i * kNoiseThreads * kNoiseCluster;
+        long long sum[2][2];  // [patch][red/blue, green]
 #pragma unroll 1
-                for (int k = 0; k < 9; ++k) {
-                    double v;
-                    if (ch == 0) {
-                        v = noise_sample(x, sigma, dwl, level, t, 27 * q + k);
-                    } else {
-                        v = __dmul_rn(0.5, __dadd_rn(noise_sample(x, sigma, dwl, level, t, 27 * q + 9 + 2 * k),
-                                                     noise_sample(x, sigma, dwl, level, t, 27 * q + 10 + 2 * k)));
-                    }
-                    if (q == 0) v1[k] = v;
-                    s = __dadd_rn(s, v);
-                }
-                mean[ch][q] = __ddiv_rn(s, 9.0);
-            }
-            double ss = 0.0;
-#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            long long srb = 0, sg = 0;
+            unsigned long long qrb = 0, qg = 0;
+#pragma unroll 1
             for (int k = 0; k < 9; ++k) {
-                const double d = __dadd_rn(v1[k], -mean[ch][0]);
-                ss = __dadd_rn(ss, __dmul_rn(d, d));
+                const int v = noise_sample(n, t, 27 * q + k);
+                const int gr = noise_sample(n, t, 27 * q + 9 + 2 * k) + noise_sample(n, t, 27 * q + 10 + 2 * k);
+                srb += v;
+                sg += gr;
+                qrb += (unsigned long long)((long long)v * v);
+                qg += (unsigned long long)((long long)gr * gr);
             }
-            var1[ch] = __ddiv_rn(ss, 9.0);
+            if (q == 0) {
+                acc[0] += 9ull * qrb - (unsigned long long)(srb * srb);
+                acc[1] += 9ull * qg - (unsigned long long)(sg * sg);
+                sum[0][0] = srb; sum[0][1] = sg;
+            } else {
+                sum[1][0] = srb; sum[1][1] = sg;
+            }
         }
-        acc[0] = __dadd_rn(acc[0], var1[0]);
-        acc[1] = __dadd_rn(acc[1], var1[1]);
-        const double d0 = __dadd_rn(mean[0][0], -mean[0][1]), d1 = __dadd_rn(mean[1][0], -mean[1][1]);
-        acc[2] = __dadd_rn(acc[2], __dmul_rn(d0, d0));
-        acc[3] = __dadd_rn(acc[3], __dmul_rn(d1, d1));
+        const long long d0 = sum[0][0] - sum[1][0], d1 = sum[0][1] - sum[1][1];
+        acc[2] += (unsigned long long)(d0 * d0);
+        acc[3] += (unsigned long long)(d1 * d1);
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) red[k][threadIdx.x] = acc[k];
-    __syncthreads();
-    for (int m = kNoiseThreads / 2; m > 0; m >>= 1) {
-        if (threadIdx.x < m)
+    for (int k = 0; k < 4; ++k) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + m];
-        __syncthreads();
+        for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = acc[k];
     }
-    if (threadIdx.x == 0)
-        table[level] = make_float4((float)(red[0][0] / kNoiseTrials), (float)(red[1][0] / kNoiseTrials),
-                                   (float)(red[2][0] / kNoiseTrials), (float)(red[3][0] / kNoiseTrials));
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    if (cluster.block_rank() == 0 && threadIdx.x < 4) {
+        unsigned long long s = 0;
+        for (int r = 0; r < kNoiseCluster; ++r) {
+            const unsigned long long *other = cluster.map_shared_rank(&red[0][0], r);
+            for (int w = 0; w < kNoiseThreads / 32; ++w) s += other[w * 4 + threadIdx.x];
+        }
+        const double scale = 81.0 * kNoiseTrials * ((threadIdx.x & 1) ? 4.0 : 1.0);
+        reinterpret_cast<float *>(table + n.level)[threadIdx.x] = (float)((double)s / scale);
+    }
+    cluster.sync();  // the other blocks' shared memory stays until it has been read
 }
 
 // piecewise-linear parameter between its value at SNR 6 (low) and at SNR 30 (high)
@@ -193,7 +230,7 @@ hmfsr_status hmfsr_noise_table(float noise_a, float noise_b, int white_level, fl
     if (!table_dev || (reinterpret_cast<uintptr_t>(table_dev) & 15) || !isfinite(noise_a) || !isfinite(noise_b) ||
         noise_a < 0.f || noise_b < 0.f || white_level < 1 || white_level > 65535)
         return HMFSR_ERR_INVALID_ARG;
-    k_noise_table<<<kNoiseLevels, kNoiseThreads, 0, (cudaStream_t)stream>>>(noise_a, noise_b, white_level,
+    k_noise_table<<<kNoiseLevels * kNoiseCluster, kNoiseThreads, 0, (cudaStream_t)stream>>>(noise_a, noise_b, white_level,
                                                                           reinterpret_cast<float4 *>(table_dev));
     return cudaGetLastError() == cudaSuccess ? HMFSR_OK : HMFSR_ERR_CUDA;
 }
