@@ -13,7 +13,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB_PATH = os.path.join(PKG, "libhmfsr.so")
 SOURCES = ("api.cu", "align.cu", "align_t4.cu", "align_t8.cu", "align_t16.cu", "align_t32.cu", "merge.cu",
-           "merge_bwd.cu", "batch.cu", "merge_static.cu", "tuning.cu", "probe.cu")
+           "merge_bwd.cu", "merge_bwd_region.cu", "batch.cu", "merge_static.cu", "tuning.cu", "probe.cu")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # -fmad=false: no automatic FMA contraction, so a device function gives the same bits in
 # every kernel it is inlined into (fused multiply-adds are written out with fmaf)

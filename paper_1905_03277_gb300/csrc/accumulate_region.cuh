@@ -79,7 +79,7 @@ constexpr int kTexP = 12;   // pitch of the staged planes of single words (8 x 4
 constexpr int kRawP = 18;   // pitch of a staged raw row's even (or odd) samples
 constexpr int kRawH = 2 * kTexN;
 constexpr int kRawOdd = kRawH * kRawP;  // the odd samples' plane follows the even one's
-constexpr int kRing = 16;               // frames whose constants are held
+constexpr int kRing = 8;                // frames whose constants are held
 
 // One frame's constants of one phase along one axis, pairs doubled for the packed operations
 struct AxisTab {
@@ -168,60 +168,62 @@ __host__ __device__ constexpr int region_items() {
     return 32 * RegionScale<SN, SD>::S * (RegionScale<SN, SD>::S / NPX);
 }
 
-// Items [item0, item0 + NT) of region (bx, by), all frames.  Every thread of the block calls this.
-// NPX x phases per thread share their Omega cell and window where they fall on the same ones
-// (fewer shared-memory reads, more registers); the results do not depend on it.
-template <bool kDen, int SN, int SD, int NT, int NPX, bool kChunk = false>
-__device__ __forceinline__ void merge_region(RegionSmem<RegionScale<SN, SD>::S> &sm, const uint16_t *__restrict__ burst,
-                                             const int4 *__restrict__ geo, const Geom &g,
-                                             const float4 *__restrict__ kern, const float *__restrict__ rhat_planes,
-                                             int ho, int wo, float *__restrict__ rgb, float *__restrict__ den_out,
-                                             int bx, int by, int item0, int tid, const ChunkIO &io = ChunkIO{}) {
-    constexpr int S = RegionScale<SN, SD>::S, kOff = RegionScale<SN, SD>::kOff;
-    constexpr int Q = 2 * SN, Q2 = 4 * SN;
-    constexpr float invQ = 1.f / (float)Q, inv2Q = 0.5f / (float)Q;
-    const int U0 = (bx - kOff) * 8, V0 = (by - kOff) * 8;  // the region's first texel
-    const size_t hw = (size_t)g.hh * g.wh, ntl = (size_t)g.ty * g.tx, fstride = (size_t)g.h * g.pitch;
+// cell (-1 or 0, relative to the texel) and phase in [0, 2Q) of a texel's output pixel s at F = 0
+template <int SN, int SD>
+__device__ __forceinline__ int region_phase(int s, int &c) {
+    const int P = 2 * SD * (RegionScale<SN, SD>::kOff + s) + SD - 2 * SN;
+    c = P < 0 ? -1 : 0;
+    return P < 0 ? P + 4 * SN : P;
+}
 
-    // this thread's pair: phases (sx, sy) of texels (u, v) and (u, v + 1) of the region
-    const int item = item0 + tid, pr = item & 31, phase = item >> 5;
-    const int sy = phase / (S / NPX), sx = (phase - sy * (S / NPX)) * NPX;  // phases sx .. sx + NPX - 1
-    const int v = 2 * (pr >> 3), u = pr & 7;
-    const int X = S * (U0 + u) + kOff + sx, Y = S * (V0 + v) + kOff + sy;
-    auto valid = [&](int k, int h) { return sy < S && X + k >= 0 && X + k < wo && Y + h * S >= 0 && Y + h * S < ho; };
-    const bool active = sy < S && X + NPX > 0 && X < wo && Y + S >= 0 && Y < ho;
-    // cell (-1 or 0) and phase of output pixel kOff + s of a texel at F = 0
-    auto phase_of = [](int s, int &c) {
-        const int P = 2 * SD * (kOff + s) + SD - 2 * SN;
-        c = P < 0 ? -1 : 0;
-        return P < 0 ? P + Q2 : P;
-    };
+// The staging of a region's frames in shared memory by the NT threads of a block.  Who stages
+// what: texels the first 121 threads, Rhat and the cross products the next warps where there are
+// enough, raw words from the last thread down.
+// kHold: a thread's raw samples wait for their turn in registers, else in shared memory as they are
+template <int SN, int SD, int NT, bool kHold>
+struct RegionStage {
+    static constexpr int S = RegionScale<SN, SD>::S, kOff = RegionScale<SN, SD>::kOff;
+    static constexpr int Q = 2 * SN, Q2 = 4 * SN;
+    static constexpr int kTexT = kTexN * kTexN, kRawT = kTexN * kRawH;
+    static constexpr int kRawL = (kRawT + NT - 1) / NT, kTexL = (kTexT + NT - 1) / NT, kNext = NT >= 256 ? 128 : 0;
+    using Smem = RegionSmem<S>;
+    Smem &sm;
+    const uint16_t *burst;
+    const int4 *geo_r;
+    const Geom &g;
+    const float4 *kern;
+    const float *rhat_planes;
+    int U0, V0, tid;
+    int tso[kTexL], tgo[kTexL], rgo[kTexL], cso[kTexL], wso[kRawL], wgo[kRawL];
+    uint32_t held[kHold ? kRawL : 1];
 
-    // ---- staging: who stages what ---------------------------------------------------------
-    // texels (and their derived terms) the first 121 threads, Rhat the next warps where there
-    // are enough, raw words from the last thread down
-    constexpr int kTexT = kTexN * kTexN, kRawT = kTexN * kRawH;
-    constexpr int kRawL = (kRawT + NT - 1) / NT, kTexL = (kTexT + NT - 1) / NT, kRh0 = NT >= 256 ? 128 : 0;
-    int tso[kTexL], tgo[kTexL], rso[kTexL], rgo[kTexL], wso[kRawL], wgo[kRawL];
+    __device__ __forceinline__ RegionStage(Smem &sm_, const uint16_t *burst_, const int4 *geo, const Geom &g_,
+                                           const float4 *kern_, const float *rhat_, int bx, int by, int tid_)
+        : sm(sm_), burst(burst_), g(g_), kern(kern_), rhat_planes(rhat_), U0((bx - kOff) * 8), V0((by - kOff) * 8),
+          tid(tid_) {
+        geo_r = geo + (size_t)clampi(2 * V0 / g.tile, 0, g.ty - 1) * g.tx + clampi(2 * U0 / g.tile, 0, g.tx - 1);
 #pragma unroll
-    for (int k = 0; k < kTexL; ++k) {
-        const int i = tid + k * NT, r = i / kTexN, c = i - r * kTexN;
-        tso[k] = i < kTexT ? i : -1;
-        tgo[k] = r * g.wh + c;
-        const int j = tid - kRh0 + k * NT, rr = j / kTexN, rc = j - rr * kTexN;
-        rso[k] = j >= 0 && j < kTexT ? rr * kTexP + rc : -1;
-        rgo[k] = clampi(V0 - 1 + rr, 0, g.hh - 1) * g.wh + clampi(U0 - 1 + rc, 0, g.wh - 1);
-        keep(tso[k]); keep(tgo[k]); keep(rso[k]); keep(rgo[k]);
-    }
+        for (int k = 0; k < kTexL; ++k) {
+            const int i = tid + k * NT, r = i / kTexN, c = i - r * kTexN;
+            tso[k] = i < kTexT ? i : -1;
+            tgo[k] = r * g.wh + c;
+            const int j = i - kNext, rr = j / kTexN, rc = j - rr * kTexN;
+            rgo[k] = clampi(V0 - 1 + rr, 0, g.hh - 1) * g.wh + clampi(U0 - 1 + rc, 0, g.wh - 1);
+            cso[k] = j >= 0 && j < kTexT ? j | (rr * kTexP + rc) << 8 : -1;  // texel | index in the planes << 8
+            keep(tso[k]); keep(tgo[k]); keep(rgo[k]); keep(cso[k]);
+        }
 #pragma unroll
-    for (int k = 0; k < kRawL; ++k) {
-        const int i = NT - 1 - tid + k * NT, r = i / kTexN, c = i - r * kTexN;
-        wso[k] = i < kRawT ? r * kRawP + c : -1;
-        wgo[k] = r * g.pitch + 2 * c;
-        keep(wso[k]); keep(wgo[k]);
+        for (int k = 0; k < kRawL; ++k) {
+            const int i = NT - 1 - tid + k * NT, r = i / kTexN, c = i - r * kTexN;
+            wso[k] = i < kRawT ? r * kRawP + c : -1;
+            wgo[k] = r * g.pitch + 2 * c;
+            keep(wso[k]); keep(wgo[k]);
+        }
     }
-    auto fill = [&](int first, int count) {
-        const int4 *geo_r = geo + (size_t)clampi(2 * V0 / g.tile, 0, g.ty - 1) * g.tx + clampi(2 * U0 / g.tile, 0, g.tx - 1);
+    // the constants of frames [first, first + count) of the accumulation order
+    __device__ __forceinline__ void fill(int first, int count) {
+        constexpr float invQ = 1.f / (float)Q, inv2Q = 0.5f / (float)Q;
+        const size_t hw = (size_t)g.hh * g.wh, ntl = (size_t)g.ty * g.tx, fstride = (size_t)g.h * g.pitch;
         for (int i = tid; i < count * 2 * S; i += NT) {
             const int it = first + i / (2 * S), k = i % (2 * S), f = frame_of_step(it, g.ref);
             const int4 e = HMFSR_LDG(geo_r + (size_t)f * ntl);
@@ -230,7 +232,7 @@ __device__ __forceinline__ void merge_region(RegionSmem<RegionScale<SN, SD>::S> 
             const bool isy = k >= S;
             const float z = __int_as_float(isy ? e.w : e.z);
             int c;
-            int p = phase_of(isy ? k - S : k, c) + ((isy ? e.y : e.x) & 63);
+            int p = region_phase<SN, SD>(isy ? k - S : k, c) + ((isy ? e.y : e.x) & 63);
             if (p >= Q2) { p -= Q2; ++c; }
             const bool hi = p >= Q;
             const float d0 = ((float)(SN - p + (hi ? Q : 0)) - z) * invQ, dm = d0 - 1.f, dp = d0 + 1.f;
@@ -243,7 +245,7 @@ __device__ __forceinline__ void merge_region(RegionSmem<RegionScale<SN, SD>::S> 
             a.q = make_float4(fr * f1, f1 * f1, fr * fr,
                               __int_as_float((c + 1) | (hi ? 256 : 0) | (in ? 0 : 512)));
             if (k == 0) {
-                typename RegionSmem<S>::Desc &d = sm.desc[it & (kRing - 1)];
+                typename Smem::Desc &d = sm.desc[it & (kRing - 1)];
                 const ptrdiff_t o = (ptrdiff_t)f * (ptrdiff_t)hw;
                 d.tex = kern + o + (in ? (ptrdiff_t)cy * g.wh + cx : 0);
                 d.raw = burst + (size_t)f * fstride + (in ? (ptrdiff_t)2 * cy * g.pitch + 2 * cx : 0);
@@ -252,10 +254,10 @@ __device__ __forceinline__ void merge_region(RegionSmem<RegionScale<SN, SD>::S> 
                 d.cy = cy;
             }
         }
-    };
-    auto desc = [&](int it) -> const typename RegionSmem<S>::Desc & { return sm.desc[it & (kRing - 1)]; };
-    auto stage_tex = [&](float4 *dst, int it) {
-        const typename RegionSmem<S>::Desc &d = desc(it);
+    }
+    __device__ __forceinline__ const typename Smem::Desc &desc(int it) const { return sm.desc[it & (kRing - 1)]; }
+    __device__ __forceinline__ void stage_tex(float4 *dst, int it) {
+        const typename Smem::Desc &d = desc(it);
         if (d.cx == INT_MIN) {
             const float4 *p = d.tex;
 #pragma unroll
@@ -267,49 +269,51 @@ __device__ __forceinline__ void merge_region(RegionSmem<RegionScale<SN, SD>::S> 
                 copy16(dst + i, d.tex + (clampi(d.cy + r, 0, g.hh - 1) * g.wh + clampi(d.cx + c, 0, g.wh - 1)));
             }
         }
-    };
-    auto stage_rhat = [&](float *dst, int it) {
+    }
+    __device__ __forceinline__ void stage_rhat(float *dst, int it) {
         if (it == 0) return;  // the base frame
         const float *p = desc(it).rh;
 #pragma unroll
         for (int k = 0; k < kTexL; ++k)
-            if (rso[k] >= 0) copy4(dst + rso[k], p + rgo[k]);
-    };
-    auto load_raw = [&](uint32_t (&w)[kRawL], int it) {
-        const typename RegionSmem<S>::Desc &d = desc(it);
+            if (cso[k] >= 0) copy4(dst + (cso[k] >> 8), p + rgo[k]);
+    }
+    // pairs of raw samples, as they are, into registers or the even plane; spread_raw turns a thread's
+    // own pairs into the two planes once they have arrived.  Registers cost less at the shared-memory
+    // path (merging at scale 1, which that path bounds: 916 us against 931 at 12 MP x 8), shared
+    // memory where registers are short (3/2: 1947 us against 1960; the adjoint, which spilled).
+    __device__ __forceinline__ void stage_raw(float *dst, int it) {
+        const typename Smem::Desc &d = desc(it);
         const uint16_t *p = d.raw;
         if (d.cx == INT_MIN) {
 #pragma unroll
             for (int k = 0; k < kRawL; ++k)
-                if (wso[k] >= 0) w[k] = HMFSR_LDG(reinterpret_cast<const uint32_t *>(p + wgo[k]));
+                if (wso[k] >= 0) {
+                    if (kHold) held[k] = HMFSR_LDG(reinterpret_cast<const uint32_t *>(p + wgo[k]));
+                    else copy4(dst + wso[k], reinterpret_cast<const float *>(p + wgo[k]));
+                }
         } else {
 #pragma unroll
             for (int k = 0; k < kRawL; ++k) {
                 const int i = NT - 1 - tid + k * NT, r = i / kTexN, c = i - r * kTexN;
-                if (i < kRawT)
-                    w[k] = HMFSR_LDG(reinterpret_cast<const uint32_t *>(
-                        p + (clampi(2 * d.cy + r, 0, g.h - 1) * g.pitch + 2 * clampi(d.cx + c, 0, g.wh - 1))));
+                const uint16_t *q = p + (clampi(2 * d.cy + r, 0, g.h - 1) * g.pitch + 2 * clampi(d.cx + c, 0, g.wh - 1));
+                if (i < kRawT) {
+                    if (kHold) held[k] = HMFSR_LDG(reinterpret_cast<const uint32_t *>(q));
+                    else copy4(dst + wso[k], reinterpret_cast<const float *>(q));
+                }
             }
         }
-    };
-    auto store_raw = [&](float *dst, const uint32_t (&w)[kRawL]) {
+    }
+    __device__ __forceinline__ void spread_raw(float *dst) {
 #pragma unroll
         for (int k = 0; k < kRawL; ++k)
             if (wso[k] >= 0) {
-                dst[wso[k]] = (float)(w[k] & 0xffffu);
-                dst[kRawOdd + wso[k]] = (float)(w[k] >> 16);
+                const uint32_t w = kHold ? held[k] : __float_as_uint(dst[wso[k]]);
+                dst[wso[k]] = (float)(w & 0xffffu);
+                dst[kRawOdd + wso[k]] = (float)(w >> 16);
             }
-    };
-    // who derives the cross products: the next warps where there are enough
-    constexpr int kCr0 = NT >= 256 ? 128 : 0;
-    int cso[kTexL];  // texel | index in the planes << 8
-#pragma unroll
-    for (int k = 0; k < kTexL; ++k) {
-        const int j = tid - kCr0 + k * NT, r = j / kTexN, c = j - r * kTexN;
-        cso[k] = j >= 0 && j < kTexT ? j | (r * kTexP + c) << 8 : -1;
-        keep(cso[k]);
     }
-    auto derive = [&](int b) {
+    // per texel M = delta u u^T, per cell the squared cross products
+    __device__ __forceinline__ void derive(int b) {
 #pragma unroll
         for (int k = 0; k < kTexL; ++k) {
             if (cso[k] >= 0) {
@@ -330,7 +334,67 @@ __device__ __forceinline__ void merge_region(RegionSmem<RegionScale<SN, SD>::S> 
                 sm.fr[b].om[tso[k]] = make_float4(t0.x, my * t0.w, -2.f * (my * t0.z), t0.y * t0.z * t0.z);
             }
         }
-    };
+    }
+    // the first frame whole, the second's texels
+    __device__ __forceinline__ void begin(int it0) {
+        fill(it0, min(kRing, g.n - it0));
+        __syncthreads();
+        stage_tex(sm.tex[it0 & 1], it0);
+        stage_rhat(sm.fr[it0 & 1].rh, it0);
+        stage_raw(sm.fr[it0 & 1].raw, it0);
+        if (it0 + 1 < g.n) stage_tex(sm.tex[(it0 + 1) & 1], it0 + 1);
+        copy_wait();
+        spread_raw(sm.fr[it0 & 1].raw);
+        __syncthreads();
+        derive(it0 & 1);
+        __syncthreads();
+    }
+    // while frame `it` is worked on (and the constants of kLag frames before it may still be read):
+    // the next frame's copies and derived terms
+    template <int kLag = 0>
+    __device__ __forceinline__ void ahead(int it, int it0) {
+        const int b = it & 1;
+        if (it + 1 >= g.n) return;
+        stage_raw(sm.fr[b ^ 1].raw, it + 1);
+        stage_rhat(sm.fr[b ^ 1].rh, it + 1);
+        if (it + 2 < g.n) stage_tex(sm.tex[b], it + 2);
+        derive(b ^ 1);
+        // frames up to it + 2 are in use, and from it - kLag on: the slots half a ring on are free
+        constexpr int kBatch = kRing / 2 - kLag;
+        static_assert((kBatch & (kBatch - 1)) == 0 && kRing / 2 >= 4, "a batch ends before frame it - kLag's slot");
+        const int next = it + kRing / 2;
+        if (next >= it0 + kRing && (it - it0) % kBatch == 0 && next < g.n) fill(next, min(kBatch, g.n - next));
+    }
+    // after it: the raw samples into place, and the block in step
+    __device__ __forceinline__ void advance(int it) {
+        if (it + 1 >= g.n) return;
+        copy_wait();
+        spread_raw(sm.fr[(it & 1) ^ 1].raw);
+        __syncthreads();
+    }
+};
+
+// Items [item0, item0 + NT) of region (bx, by), all frames.  Every thread of the block calls this.
+// NPX x phases per thread share their Omega cell and window where they fall on the same ones
+// (fewer shared-memory reads, more registers); the results do not depend on it.
+template <bool kDen, int SN, int SD, int NT, int NPX, bool kChunk = false>
+__device__ __forceinline__ void merge_region(RegionSmem<RegionScale<SN, SD>::S> &sm, const uint16_t *__restrict__ burst,
+                                             const int4 *__restrict__ geo, const Geom &g,
+                                             const float4 *__restrict__ kern, const float *__restrict__ rhat_planes,
+                                             int ho, int wo, float *__restrict__ rgb, float *__restrict__ den_out,
+                                             int bx, int by, int item0, int tid, const ChunkIO &io = ChunkIO{}) {
+    constexpr int S = RegionScale<SN, SD>::S, kOff = RegionScale<SN, SD>::kOff;
+    constexpr float inv2Q = 0.25f / (float)SN;
+    const int U0 = (bx - kOff) * 8, V0 = (by - kOff) * 8;  // the region's first texel
+
+    // this thread's pair: phases (sx, sy) of texels (u, v) and (u, v + 1) of the region
+    const int item = item0 + tid, pr = item & 31, phase = item >> 5;
+    const int sy = phase / (S / NPX), sx = (phase - sy * (S / NPX)) * NPX;  // phases sx .. sx + NPX - 1
+    const int v = 2 * (pr >> 3), u = pr & 7;
+    const int X = S * (U0 + u) + kOff + sx, Y = S * (V0 + v) + kOff + sy;
+    auto valid = [&](int k, int h) { return sy < S && X + k >= 0 && X + k < wo && Y + h * S >= 0 && Y + h * S < ho; };
+    const bool active = sy < S && X + NPX > 0 && X < wo && Y + S >= 0 && Y < ho;
+    RegionStage<SN, SD, NT, SN == SD> st(sm, burst, geo, g, kern, rhat_planes, bx, by, tid);
 
     PixelAcc none;
     none.mR = none.mG = none.mB = 0.f;  // the first frame's exponents are -q'; it then sets the shifts
@@ -364,42 +428,20 @@ __device__ __forceinline__ void merge_region(RegionSmem<RegionScale<SN, SD>::S> 
     bool big = fresh || shifts_big();
     float rfx[NPX], rfy;
     int ro[NPX], rcx, rcy;
-    rfy = (float)phase_of(sy, rcy) * inv2Q;
+    rfy = (float)region_phase<SN, SD>(sy, rcy) * inv2Q;
     keep(rfy);
 #pragma unroll
     for (int k = 0; k < NPX; ++k) {
-        rfx[k] = (float)phase_of(sx + k, rcx) * inv2Q;
+        rfx[k] = (float)region_phase<SN, SD>(sx + k, rcx) * inv2Q;
         ro[k] = (v + 1 + rcy) * kTexP + u + 1 + rcx;  // Rhat cell in shared memory
         keep(rfx[k]); keep(ro[k]);
     }
     int o0 = v * kTexP + u, m0 = v * kTexN + u, w0 = 2 * v * kRawP + u, txo = sx, tyo = S + sy, act = active ? 1 : 0;
     keep(o0); keep(m0); keep(w0); keep(txo); keep(tyo); keep(act);
-    if (it0 < g.n) {
-        fill(it0, min(kRing, g.n - it0));
-        __syncthreads();
-        stage_tex(sm.tex[it0 & 1], it0);
-        stage_rhat(sm.fr[it0 & 1].rh, it0);
-        uint32_t w[kRawL];
-        load_raw(w, it0);
-        if (it0 + 1 < g.n) stage_tex(sm.tex[(it0 + 1) & 1], it0 + 1);
-        store_raw(sm.fr[it0 & 1].raw, w);
-        copy_wait();
-        __syncthreads();
-        derive(it0 & 1);
-        __syncthreads();
-    }
+    if (it0 < g.n) st.begin(it0);
     for (int it = it0; it < g.n; ++it) {
         const int b = it & 1;
-        uint32_t w[kRawL];
-        if (it + 1 < g.n) {
-            load_raw(w, it + 1);
-            stage_rhat(sm.fr[b ^ 1].rh, it + 1);
-            if (it + 2 < g.n) stage_tex(sm.tex[b], it + 2);
-            derive(b ^ 1);
-            // the slots of the frames before this one are free: refill them half a ring at a time
-            if (it > it0 && (it - it0) % (kRing / 2) == 0 && it + kRing / 2 < g.n)
-                fill(it + kRing / 2, min(kRing / 2, g.n - it - kRing / 2));
-        }
+        st.ahead(it, it0);
         do {  // left early where the frame adds nothing
             if (!act) break;
             const typename RegionSmem<S>::Frame &fr = sm.fr[b];
@@ -523,7 +565,7 @@ __device__ __forceinline__ void merge_region(RegionSmem<RegionScale<SN, SD>::S> 
                     }
                 }
                 if (kx[k] & 512) {  // samples outside the frame are left out
-                    const typename RegionSmem<S>::Desc &d = desc(it);
+                    const typename RegionSmem<S>::Desc &d = st.desc(it);
                     const int ax = 2 * (d.cx + u + (kx[k] & 255)) + (hix ? 1 : 0), ay = 2 * (d.cy + v + (ky & 255)) + (hiy ? 1 : 0);
 #pragma unroll
                     for (int j = 0; j < 3; ++j)
@@ -624,11 +666,7 @@ __device__ __forceinline__ void merge_region(RegionSmem<RegionScale<SN, SD>::S> 
                 }
             }
         } while (false);
-        if (it + 1 < g.n) {
-            store_raw(sm.fr[b ^ 1].raw, w);
-            copy_wait();
-            __syncthreads();
-        }
+        st.advance(it);
     }
     const size_t po = (size_t)ho * wo;
 #pragma unroll

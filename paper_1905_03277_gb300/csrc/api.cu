@@ -276,9 +276,7 @@ size_t hmfsr_workspace_size(int op, const hmfsr_burst_desc *desc, int tile, int 
         if (!valid_scale(scale_num, scale_den)) return 0;
         MergePlanes P;
         BwdPlanes B;
-        const int ho = (int)(((long long)desc->height * scale_num) / scale_den);
-        const int wo = (int)(((long long)desc->width * scale_num) / scale_den);
-        return carve_backward(nullptr, g, ho, wo, carve_merge(nullptr, g, &P), &B);
+        return carve_backward(nullptr, g, scale_num, scale_den, carve_merge(nullptr, g, &P), &B);
     }
     return 0;
 }
@@ -606,13 +604,11 @@ hmfsr_status merge_backward_impl(const uint16_t *burst_dev, const hmfsr_burst_de
     Geom g = make_geom(desc, params->tile);
     MergePlanes P;
     BwdPlanes B;
-    const int ho = (int)(((long long)desc->height * scale_num) / scale_den);
-    const int wo = (int)(((long long)desc->width * scale_num) / scale_den);
     const size_t fwd = carve_merge(nullptr, g, &P);
-    hmfsr_status st = check_ws(ws, ws_bytes, carve_backward(nullptr, g, ho, wo, fwd, &B));
+    hmfsr_status st = check_ws(ws, ws_bytes, carve_backward(nullptr, g, scale_num, scale_den, fwd, &B));
     if (st != HMFSR_OK) return st;
     carve_merge(ws, g, &P);
-    carve_backward(ws, g, ho, wo, fwd, &B);
+    carve_backward(ws, g, scale_num, scale_den, fwd, &B);
     cudaStream_t s = (cudaStream_t)stream;
     const MergeConsts c = consts_of(params);
     SideStream *side = side_stream();
@@ -635,8 +631,8 @@ hmfsr_status merge_backward_impl(const uint16_t *burst_dev, const hmfsr_burst_de
     e[9] = cudaStreamWaitEvent(s, side->join, 0);
     for (cudaError_t x : e)
         if (x != cudaSuccess) return HMFSR_ERR_CUDA;
-    if (launch_bwd_main(burst_dev, motion_dev, g, c, P, B, scale_num, scale_den, rgb_dev, den_dev, grad_rgb_dev, s) !=
-            cudaSuccess ||
+    if (launch_bwd_main(burst_dev, motion_dev, g, c, P, B, scale_num, scale_den, rgb_dev, den_dev, grad_rgb_dev,
+                        s) != cudaSuccess ||
         cudaStreamWaitEvent(s, side->fork, 0) != cudaSuccess)
         return HMFSR_ERR_CUDA;
     return cuda_status(launch_bwd_finish(g, B, scale_num, scale_den, grad_params_dev, grad_motion_dev, s));

@@ -230,6 +230,8 @@ cudaError_t launch_merge_accum(const uint16_t *burst, const float *motion, const
 cudaError_t launch_merge_accum_chunk(const uint16_t *burst, const float *motion, const Geom &g, const MergePlanes &P,
                                      int snum, int sden, float *rgb, float *den, const float *state_in,
                                      float *state_out, bool skip_base, cudaStream_t s);
+// the window geometry of every (frame, tile) for an output scale, into P.geo
+cudaError_t launch_geo(const float *motion, const Geom &g, const MergePlanes &P, int snum, int sden, cudaStream_t s);
 cudaError_t launch_export_stages(const Geom &g, const MergePlanes &P, float *omega, float *rhat, cudaStream_t s);
 
 // adjoint of the merge: buffers beyond the forward planes
@@ -245,9 +247,25 @@ struct BwdPlanes {
     double *part6;          // [n_bwd_blocks][6] kernel-parameter partial sums
     double *part2;          // [n_rp_blocks][2] (s2, t) partial sums
     unsigned char *sel;     // [n][ty*tx] 1 where the motion prior chose s2
+    // the region kernels (merge_bwd_region.cu) instead of the *_pix, *_rows and *_tex planes above:
+    float *rhbar_phase;     // [n][S*S phases][half-res grid] dL/dRhat at output pixels, by phase
+    float2 *vbar_region;    // [n][regions][phases]{x, y} motion contributions through the weights, with rounding errors
+    float2 *vbar_block;     // [n][8 x 8-texel blocks] motion contributions through R
     int n_bwd_blocks, n_rp_blocks;
 };
-size_t carve_backward(void *ws, const Geom &g, int ho, int wo, size_t fwd_bytes, BwdPlanes *B);
+size_t carve_backward(void *ws, const Geom &g, int snum, int sden, size_t fwd_bytes, BwdPlanes *B);
+// the adjoint by regions (scales 1, 3/2 and 2, tiles of 16 px and more)
+bool bwd_region(const Geom &g, int snum, int sden);
+cudaError_t launch_bwd_region_main(const uint16_t *burst, const float *motion, const Geom &g, const MergeConsts &c,
+                                   const MergePlanes &P, const BwdPlanes &B, int snum, int sden, const float *rgb,
+                                   const float *lden, const float *grad_rgb, cudaStream_t s);
+cudaError_t launch_bwd_region_finish(const Geom &g, const BwdPlanes &B, int snum, int sden, float *grad_motion,
+                                     cudaStream_t s);
+struct BwdRegionSizes {
+    size_t rhbar, vregion, vblock;  // elements
+    int bwd_blocks, rp_blocks;
+};
+BwdRegionSizes bwd_region_sizes(const Geom &g, int snum, int sden);
 // the adjoint's four parts (merge_bwd.cu): shape, then robust (after the preparation),
 // main (after shape and the preparation), finish (after robust and main)
 cudaError_t launch_bwd_shape(const uint16_t *burst, const Geom &g, const BwdPlanes &B, cudaStream_t s);

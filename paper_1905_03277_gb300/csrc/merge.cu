@@ -287,15 +287,21 @@ cudaError_t launch_merge_prep(const uint16_t *burst, const float *motion, const 
     return launch_merge_prep_motion(motion, g, c, P, s);
 }
 
+cudaError_t launch_geo(const float *motion, const Geom &g, const MergePlanes &P, int snum, int sden, cudaStream_t s) {
+    const int ntl = g.ty * g.tx;
+    k_geo<<<div_up(g.n * ntl, 128), 128, 0, s>>>(reinterpret_cast<const float2 *>(motion), g.n, ntl, g.ref,
+                                                 stage::geo_q(g.tile, snum, sden), P.geo,
+                                                 stage::region_kind(g.tile, snum, sden) != 0);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_merge_accum(const uint16_t *burst, const float *motion, const Geom &g, const MergePlanes &P,
                                int snum, int sden, float *rgb, float *den, cudaStream_t s) {
     StageRange range("hmfsr merge: accumulation and normalisation");
     CheckedLaunches checked(s);
     const int ho = (int)(((long long)g.h * snum) / sden), wo = (int)(((long long)g.w * snum) / sden);
-    const int ntl = g.ty * g.tx;
-    k_geo<<<div_up(g.n * ntl, 128), 128, 0, s>>>(reinterpret_cast<const float2 *>(motion), g.n, ntl, g.ref,
-                                                 stage::geo_q(g.tile, snum, sden), P.geo,
-                                                 stage::region_kind(g.tile, snum, sden) != 0);
+    const cudaError_t e = launch_geo(motion, g, P, snum, sden, s);
+    if (e != cudaSuccess) return e;
     if (den)
         launch_k_merge<true, false>(s, burst, g, P, snum, sden, ho, wo, rgb, den, stage::ChunkIO{});
     else
@@ -309,10 +315,8 @@ cudaError_t launch_merge_accum_chunk(const uint16_t *burst, const float *motion,
     StageRange range("hmfsr merge: accumulation of one chunk of frames");
     CheckedLaunches checked(s);
     const int ho = (int)(((long long)g.h * snum) / sden), wo = (int)(((long long)g.w * snum) / sden);
-    const int ntl = g.ty * g.tx;
-    k_geo<<<div_up(g.n * ntl, 128), 128, 0, s>>>(reinterpret_cast<const float2 *>(motion), g.n, ntl, g.ref,
-                                                 stage::geo_q(g.tile, snum, sden), P.geo,
-                                                 stage::region_kind(g.tile, snum, sden) != 0);
+    const cudaError_t e = launch_geo(motion, g, P, snum, sden, s);
+    if (e != cudaSuccess) return e;
     stage::ChunkIO io;
     io.state_in = state_in;
     io.state_out = state_out;

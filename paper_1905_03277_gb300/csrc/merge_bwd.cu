@@ -8,77 +8,13 @@
 // log2 of its weight sum are read back, so each sample's normalised weight is
 // 2^-(q' + log2 den).  All reductions are deterministic: per-pixel and per-texel
 // contributions go to buffers and are summed in a fixed order in FP64.
-#include "hmfsr_internal.cuh"
+#include "adjoint_common.cuh"
 
 namespace hmfsr {
 namespace {
 
 constexpr float kHalfLog2e = 0.72134752044448170368f;  // log2(e) / 2
 constexpr int kBwdW = 32, kBwdH = 4, kBwdThreads = kBwdW * kBwdH;
-
-// Block sums in a fixed order without FP64 arithmetic per element (FP64 is scarce on this
-// GPU): each warp adds its lanes' values by butterflies carrying the exact rounding error
-// of every FP32 addition (two-sum), lane 0 stores the warp's (sum, error) pair; the
-// caller's thread 0 then adds the warps' pairs in FP64 in warp order.
-template <int K>
-__device__ __forceinline__ void warp_sums_comp(float (&v)[K], float (&e)[K]) {
-#pragma unroll
-    for (int q = 0; q < K; ++q) e[q] = 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int q = 0; q < K; ++q) {
-            const float a = v[q], b = __shfl_xor_sync(0xffffffffu, v[q], o);
-            const float t = a + b, bp = t - a;
-            const float err = (a - (t - bp)) + (b - bp);
-            e[q] = (e[q] + __shfl_xor_sync(0xffffffffu, e[q], o)) + err;
-            v[q] = t;
-        }
-}
-
-// The six kernel parameters' contribution of one texel.  With k_x = s_x^2 the kernel
-// variances of Eq. 4 / S.1 (s_along, s_across their square roots), d k_x / d p_q = 2 s_x
-// a_x[q], and the texel adds sum_q (d k_across / d p_q bo1 + d k_along / d p_q bo2) to
-// pb[q], bo1 and bo2 being dL/dk_across and dL/dk_along times the bilinear weight:
-//   a_along  = {(1-D) k_stretch A + D k_denoise, D k_detail, (kd - kh_al) dD/dD_th,
-//               (kd - kh_al) dD/dD_tr, (1-D) k_detail A, 0},
-//   a_across = {(1-D) / (k_shrink A) + D k_denoise, D k_detail, (kd - kh_ac) dD/dD_th,
-//               (kd - kh_ac) dD/dD_tr, 0, -(1-D) k_detail / (k_shrink^2 A)}
-// with kd = k_detail k_denoise, kh_al = k_detail k_stretch A, kh_ac = k_detail /
-// (k_shrink A), D = clamp(1 - sqrt(l1_norm) / D_tr + D_th, 0, 1) and its derivatives 0
-// where clamped.  Per-call constants in KConsts; 1/A on the SFU.
-struct KConsts {
-    float inv_dtr, inv_shrink, kd, kds, kdi, kdi2;
-};
-__device__ __forceinline__ KConsts kconsts_of(const MergeConsts &c) {
-    KConsts k;
-    k.inv_dtr = 1.f / c.d_tr;
-    k.inv_shrink = 1.f / c.k_shrink;
-    k.kd = c.k_detail * c.k_denoise;
-    k.kds = c.k_detail * c.k_stretch;
-    k.kdi = c.k_detail * k.inv_shrink;
-    k.kdi2 = k.kdi * k.inv_shrink;
-    return k;
-}
-__device__ __forceinline__ void kernel_grad_acc(const float4 sh, const MergeConsts &c, const KConsts &k, float bo1,
-                                                float bo2, float (&pb)[6]) {
-    const float A = sh.x, rl = sh.y, invA = fast_rcp(A);
-    const float Draw = 1.f - rl * k.inv_dtr + c.d_th;
-    const float D = fminf(fmaxf(Draw, 0.f), 1.f), omD = 1.f - D;
-    const bool inside = Draw > 0.f && Draw < 1.f;
-    const float kh_al = k.kds * A, kh_ac = k.kdi * invA;
-    const float s_al = omD * kh_al + D * k.kd, s_ac = omD * kh_ac + D * k.kd;
-    const float P = 2.f * s_ac * bo1, Qv = 2.f * s_al * bo2;  // dL/d(a_across), dL/d(a_along) weights
-    pb[0] = fmaf(P, omD * k.inv_shrink * invA + D * c.k_denoise, fmaf(Qv, omD * c.k_stretch * A + D * c.k_denoise, pb[0]));
-    pb[1] = fmaf(P + Qv, D * c.k_detail, pb[1]);
-    if (inside) {
-        const float sD = P * (k.kd - kh_ac) + Qv * (k.kd - kh_al);
-        pb[2] += sD;
-        pb[3] = fmaf(sD, rl * k.inv_dtr * k.inv_dtr, pb[3]);
-    }
-    pb[4] = fmaf(Qv, omD * c.k_detail * A, pb[4]);
-    pb[5] = fmaf(-P, omD * k.kdi2 * invA, pb[5]);
-}
 
 // ---------------------------------------------------------------------------------------
 // per texel: what the kernel-shape derivative needs {A, sqrt(l1_norm), cos 2t, sin 2t}
@@ -649,19 +585,22 @@ __global__ void __launch_bounds__(kRedThreads) k_motion_reduce(const float2 *__r
     }
 }
 
-__global__ void __launch_bounds__(kRedThreads) k_param_reduce(const double *__restrict__ p6, int n6,
+// 512 threads: at 128 each walked 64 partials of the fitting workload one after another (11 us)
+constexpr int kParamThreads = 512;
+
+__global__ void __launch_bounds__(kParamThreads) k_param_reduce(const double *__restrict__ p6, int n6,
                                                               const double *__restrict__ p2, int n2,
                                                               float *__restrict__ grad_params) {
-    __shared__ double s_red[kRedThreads];
+    __shared__ double s_red[kParamThreads];
     const int q = blockIdx.x, tid = threadIdx.x;  // q = 0..7
     double acc = 0.0;
     if (q < 6)
-        for (int k = tid; k < n6; k += kRedThreads) acc += p6[(size_t)k * 6 + q];
+        for (int k = tid; k < n6; k += kParamThreads) acc += p6[(size_t)k * 6 + q];
     else
-        for (int k = tid; k < n2; k += kRedThreads) acc += p2[(size_t)k * 2 + (q - 6)];
+        for (int k = tid; k < n2; k += kParamThreads) acc += p2[(size_t)k * 2 + (q - 6)];
     s_red[tid] = acc;
     __syncthreads();
-    for (int sstep = kRedThreads / 2; sstep > 0; sstep >>= 1) {
+    for (int sstep = kParamThreads / 2; sstep > 0; sstep >>= 1) {
         if (tid < sstep) s_red[tid] += s_red[tid + sstep];
         __syncthreads();
     }
@@ -671,18 +610,31 @@ __global__ void __launch_bounds__(kRedThreads) k_param_reduce(const double *__re
 }  // namespace
 
 // workspace of the adjoint beyond the forward planes
-size_t carve_backward(void *ws, const Geom &g, int ho, int wo, size_t fwd_bytes, BwdPlanes *B) {
+size_t carve_backward(void *ws, const Geom &g, int snum, int sden, size_t fwd_bytes, BwdPlanes *B) {
+    const int ho = (int)(((long long)g.h * snum) / sden), wo = (int)(((long long)g.w * snum) / sden);
     char *base = static_cast<char *>(ws);
     size_t off = fwd_bytes;
-    auto take = [&](size_t bytes) {
-        size_t o = off;
+    const auto take = [&](size_t bytes) -> void * {
+        const size_t o = off;
         off = (off + bytes + 255) & ~(size_t)255;
-        return base ? (void *)(base + o) : nullptr;
+        return base ? static_cast<void *>(base + o) : nullptr;
     };
     const size_t hw = (size_t)g.hh * g.wh, npx = (size_t)ho * wo;
     B->shape = (float4 *)take(sizeof(float4) * g.n * hw);
     B->rb = (float4 *)take(sizeof(float4) * g.n * hw);
     B->flags = (unsigned char *)take(g.n * hw);
+    B->sel = (unsigned char *)take((size_t)g.n * g.ty * g.tx);
+    if (bwd_region(g, snum, sden)) {
+        const BwdRegionSizes z = bwd_region_sizes(g, snum, sden);
+        B->rhbar_phase = (float *)take(sizeof(float) * z.rhbar);
+        B->vbar_region = (float2 *)take(sizeof(float2) * z.vregion);
+        B->vbar_block = (float2 *)take(sizeof(float2) * z.vblock);
+        B->n_bwd_blocks = z.bwd_blocks;
+        B->n_rp_blocks = z.rp_blocks;
+        B->part6 = (double *)take(sizeof(double) * 6 * (size_t)B->n_bwd_blocks);
+        B->part2 = (double *)take(sizeof(double) * 2 * (size_t)B->n_rp_blocks);
+        return off;
+    }
     B->rhbar_tex = (float *)take(sizeof(float) * g.n * hw);
     B->vbar_tex = (float2 *)take(sizeof(float2) * g.n * hw);
     B->vbar_pix = (float2 *)take(sizeof(float2) * g.n * npx);
@@ -692,7 +644,6 @@ size_t carve_backward(void *ws, const Geom &g, int ho, int wo, size_t fwd_bytes,
     B->n_rp_blocks = div_up(g.wh, kRpThreads) * g.hh * g.n;
     B->part6 = (double *)take(sizeof(double) * 6 * (size_t)B->n_bwd_blocks);
     B->part2 = (double *)take(sizeof(double) * 2 * (size_t)B->n_rp_blocks);
-    B->sel = (unsigned char *)take((size_t)g.n * g.ty * g.tx);
     return off;
 }
 
@@ -720,6 +671,8 @@ cudaError_t launch_bwd_robust(const float *motion, const Geom &g, const MergeCon
 cudaError_t launch_bwd_main(const uint16_t *burst, const float *motion, const Geom &g, const MergeConsts &c,
                             const MergePlanes &P, const BwdPlanes &B, int snum, int sden, const float *rgb,
                             const float *lden, const float *grad_rgb, cudaStream_t s) {
+    if (bwd_region(g, snum, sden))
+        return launch_bwd_region_main(burst, motion, g, c, P, B, snum, sden, rgb, lden, grad_rgb, s);
     const int ho = (int)(((long long)g.h * snum) / sden), wo = (int)(((long long)g.w * snum) / sden);
     const float2 *mv = reinterpret_cast<const float2 *>(motion);
     const dim3 tex_grid(div_up(g.wh, 128), g.hh, g.n);
@@ -733,12 +686,18 @@ cudaError_t launch_bwd_main(const uint16_t *burst, const float *motion, const Ge
 
 cudaError_t launch_bwd_finish(const Geom &g, const BwdPlanes &B, int snum, int sden, float *grad_params,
                               float *grad_motion, cudaStream_t s) {
+    if (bwd_region(g, snum, sden)) {
+        const cudaError_t e = launch_bwd_region_finish(g, B, snum, sden, grad_motion, s);
+        if (e != cudaSuccess) return e;
+        k_param_reduce<<<8, kParamThreads, 0, s>>>(B.part6, B.n_bwd_blocks, B.part2, B.n_rp_blocks, grad_params);
+        return cudaGetLastError();
+    }
     const int ho = (int)(((long long)g.h * snum) / sden), wo = (int)(((long long)g.w * snum) / sden);
     k_rpath<<<dim3(div_up(g.wh, kRpThreads), g.hh, g.n), kRpThreads, 0, s>>>(B.rhbar_tex, B.flags, B.rb, g,
                                                                            B.vbar_tex, B.part2);
     k_motion_reduce<<<div_up(g.n * g.ty * g.tx, kRedThreads / 32), kRedThreads, 0, s>>>(B.vbar_pix, B.vbar_tex, g, snum,
                                                                                       sden, ho, wo, grad_motion);
-    k_param_reduce<<<8, kRedThreads, 0, s>>>(B.part6, B.n_bwd_blocks, B.part2, B.n_rp_blocks, grad_params);
+    k_param_reduce<<<8, kParamThreads, 0, s>>>(B.part6, B.n_bwd_blocks, B.part2, B.n_rp_blocks, grad_params);
     return cudaGetLastError();
 }
 
