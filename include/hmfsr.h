@@ -156,9 +156,9 @@ hmfsr_status hmfsr_merge_accumulate(const uint16_t *burst_dev, const hmfsr_burst
 
 /* Bounded-memory merge (Sec. 6 and Table 2: memory that does not grow with the frame
  * count): the same outputs, bit for bit, as hmfsr_merge with these arguments, computed
- * chunk_frames non-base frames at a time.  Each chunk's frames and the base frame are
- * copied into a packed sub-burst in the workspace, their planes (kernel covariances,
- * robustness) are prepared there, and the accumulation continues from the running sums
+ * chunk_frames non-base frames at a time.  The frames are read where they lie in the
+ * burst; a chunk's planes (kernel covariances, robustness) are prepared in the
+ * workspace, and the accumulation continues from the running sums
  * of the earlier chunks: per output pixel and channel the numerator, the denominator
  * and the exponent shift, 9 floats, kept in the workspace between chunks.  The frames
  * are merged in hmfsr_merge's order (the base frame, then the others in order), so the

@@ -193,12 +193,14 @@ __device__ __forceinline__ int floor_div_q(int a, int b) {
 // is zero: its motion is zero by definition.  i runs over n x tiles.  split: each integer F
 // comes as (F div 2Q) << 6 | F mod 2Q (a half-res cell and a phase, 2Q <= 32); motion that
 // takes every window far outside any frame is clamped to 2^26 / Q px.
-__device__ __forceinline__ void geo_entry(const float2 *__restrict__ motion, int n, int ntl, int ref, int Q,
+__device__ __forceinline__ void geo_entry(const float2 *__restrict__ motion, const Geom &g, int Q,
                                           int4 *__restrict__ geo, int i, bool split) {
-    if (i >= n * ntl) return;
+    const int ntl = g.ty * g.tx;
+    if (i >= g.n * ntl) return;
     int4 e = make_int4(0, 0, 0, 0);
-    if (i / ntl != ref) {
-        const float2 mv = HMFSR_LD(motion + i);
+    const int f = i / ntl;
+    if (f != g.ref) {
+        const float2 mv = HMFSR_LD(motion + ((size_t)src_frame(g, f) * ntl + (i - f * ntl)));
         const int FX = floor_mul(Q, mv.x), FY = floor_mul(Q, mv.y);
         const float fQ = (float)Q;
         e = make_int4(FX, FY, __float_as_int(fmaf(fQ, mv.x, -(float)FX)), __float_as_int(fmaf(fQ, mv.y, -(float)FY)));
@@ -362,7 +364,7 @@ __device__ __forceinline__ void merge_px(const uint16_t *__restrict__ burst, con
             Cy[i] = Byy * dys[i] * dys[i];
         }
         // the 3x3 Bayer neighbourhood; samples outside the frame are left out
-        const uint16_t *fr = burst + (size_t)f * fstride;
+        const uint16_t *fr = burst + (size_t)(kChunk ? src_frame(g, f) : f) * fstride;
         float q[3][3], rv[3][3];
         if ((unsigned)(kx - 1) < (unsigned)(g.w - 2) && (unsigned)(ky - 1) < (unsigned)(g.h - 2))
             gather3x3<false>(fr, g.pitch, g.h, g.w, kx, ky, Ax, Ex, Cy, dys, q, rv);
@@ -603,7 +605,7 @@ __device__ __forceinline__ void merge_quad1(const uint16_t *__restrict__ burst, 
             om.fy[pb] = ((float)(gy & 3) + zy) * 0.25f;
         }
         const int bx = X + Kx - 1, by = Y + Ky - 1;  // first sample of the raw block
-        const uint16_t *fr = burst + (size_t)f * fstride;
+        const uint16_t *fr = burst + (size_t)(kChunk ? src_frame(g, f) : f) * fstride;
         const bool inside = (unsigned)bx <= (unsigned)(g.w - 4) && (unsigned)by <= (unsigned)(g.h - NY - 2) &&
                             u + om.Ox[0] >= 0 && u + om.Ox[1] + 1 < g.wh && om.Oy[0] >= 0 &&
                             om.Oy[NY - 1] + 1 < g.hh;

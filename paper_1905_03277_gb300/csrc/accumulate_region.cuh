@@ -248,7 +248,7 @@ struct RegionStage {
                 typename Smem::Desc &d = sm.desc[it & (kRing - 1)];
                 const ptrdiff_t o = (ptrdiff_t)f * (ptrdiff_t)hw;
                 d.tex = kern + o + (in ? (ptrdiff_t)cy * g.wh + cx : 0);
-                d.raw = burst + (size_t)f * fstride + (in ? (ptrdiff_t)2 * cy * g.pitch + 2 * cx : 0);
+                d.raw = burst + (size_t)src_frame(g, f) * fstride + (in ? (ptrdiff_t)2 * cy * g.pitch + 2 * cx : 0);
                 d.rh = rhat_planes + o;
                 d.cx = in ? INT_MIN : cx;
                 d.cy = cy;

@@ -157,30 +157,23 @@ size_t carve_merge(void *ws, const Geom &g, MergePlanes *P) {
     return c.off;
 }
 
-// Bounded-memory merge workspace: a sub-burst of slots = min(n, chunk + 1) packed frames
-// (slot 0 the base frame), their motion rows, the merge planes of that sub-burst, and the
-// running sums of every output pixel (9 planes of Ho x Wo floats).
+// Bounded-memory merge workspace: the merge planes of a chunk, min(n, chunk + 1) frames (frame 0
+// the base frame), and the running sums of every output pixel (9 planes of Ho x Wo floats).
 struct ChunkLayout {
-    uint16_t *sub = nullptr;
-    float *sub_motion = nullptr;
     MergePlanes P;
     float *state = nullptr;
-    hmfsr_burst_desc sd;
-    Geom gs;
+    Geom g;  // of the chunk; its frames are read where they lie in the burst
 };
 
 size_t carve_chunked(void *ws, const hmfsr_burst_desc *d, int tile, int num, int den, int chunk, ChunkLayout *L) {
-    L->sd = *d;
-    L->sd.n_frames = d->n_frames < chunk + 1 ? d->n_frames : chunk + 1;
-    L->sd.pitch_elems = d->width;
-    L->sd.ref = 0;
-    L->gs = make_geom(&L->sd, tile);
+    L->g = make_geom(d, tile);
+    L->g.n = d->n_frames < chunk + 1 ? d->n_frames : chunk + 1;
+    L->g.ref = 0;
+    L->g.src_base = d->ref;
+    L->g.src_first = 0;
     const size_t ho = (size_t)(((long long)d->height * num) / den), wo = (size_t)(((long long)d->width * num) / den);
     Carver c(ws);
-    L->sub = c.take<uint16_t>((size_t)L->sd.n_frames * d->height * d->width);
-    L->sub_motion = c.take<float>((size_t)L->sd.n_frames * L->gs.ty * L->gs.tx * 2);
-    const size_t planes = carve_merge(ws ? static_cast<char *>(ws) + c.off : nullptr, L->gs, &L->P);
-    c.off = align_up(c.off + planes);
+    c.off = align_up(carve_merge(ws, L->g, &L->P));
     L->state = c.take<float>(9 * ho * wo);
     return c.off;
 }
@@ -424,35 +417,20 @@ hmfsr_status hmfsr_merge_chunked(const uint16_t *burst_dev, const hmfsr_burst_de
     chk.add(rgb_dev, rgb_bytes(desc, scale_num, scale_den));
     chk.add(den_dev, rgb_bytes(desc, scale_num, scale_den));
     chk.add_ws(ws, need);
-    const size_t frame_px = (size_t)desc->height * desc->width, motion_row = (size_t)g.ty * g.tx * 2;
-    // one frame of the burst into a slot of the packed sub-burst, with its motion row
-    auto put = [&](int f, int slot) -> bool {
-        const uint16_t *src = burst_dev + (size_t)f * desc->height * desc->pitch_elems;
-        if (cudaMemcpy2DAsync(L.sub + (size_t)slot * frame_px, (size_t)desc->width * 2, src,
-                              (size_t)desc->pitch_elems * 2, (size_t)desc->width * 2, desc->height,
-                              cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-            return false;
-        return cudaMemcpyAsync(L.sub_motion + (size_t)slot * motion_row, motion_dev + (size_t)f * motion_row,
-                               motion_row * sizeof(float), cudaMemcpyDeviceToDevice, s) == cudaSuccess;
-    };
-    if (!put(desc->ref, 0)) return HMFSR_ERR_CUDA;
     const int others = desc->n_frames - 1;
     const int chunks = others > 0 ? (others + chunk_frames - 1) / chunk_frames : 1;
     for (int ci = 0; ci < chunks; ++ci) {
         const int o0 = ci * chunk_frames;
         const int m = others - o0 < chunk_frames ? others - o0 : chunk_frames;
-        for (int j = 0; j < m; ++j) {
-            const int o = o0 + j, f = o < desc->ref ? o : o + 1;  // the others in order
-            if (!put(f, 1 + j)) return HMFSR_ERR_CUDA;
-        }
-        Geom gc = L.gs;
+        Geom gc = L.g;
         gc.n = 1 + (m > 0 ? m : 0);
+        gc.src_first = o0;
         // the base frame's planes (slot 0) are made by the first chunk and kept
-        if (launch_merge_prep_frames(L.sub, gc, c, L.P, s, ci > 0 ? 1 : 0) != cudaSuccess ||
-            launch_merge_prep_motion(L.sub_motion, gc, c, L.P, s) != cudaSuccess)
+        if (launch_merge_prep_frames(burst_dev, gc, c, L.P, s, ci > 0 ? 1 : 0) != cudaSuccess ||
+            launch_merge_prep_motion(motion_dev, gc, c, L.P, s) != cudaSuccess)
             return HMFSR_ERR_CUDA;
         const bool last = (ci == chunks - 1);
-        if (launch_merge_accum_chunk(L.sub, L.sub_motion, gc, L.P, scale_num, scale_den, rgb_dev, den_dev,
+        if (launch_merge_accum_chunk(burst_dev, motion_dev, gc, L.P, scale_num, scale_den, rgb_dev, den_dev,
                                      ci > 0 ? L.state : nullptr, last ? nullptr : L.state, ci > 0, s) != cudaSuccess)
             return HMFSR_ERR_CUDA;
     }

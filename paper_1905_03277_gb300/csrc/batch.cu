@@ -217,8 +217,8 @@ __device__ __forceinline__ void run_sub(const BatchBurst &b, int s, int k, int t
             break;
         }
         case S_STRENGTH:
-            stage::strength(mv, g.n, g.ty, g.tx, b.c.m_th, b.c.s1, b.c.s2, b.P.s_tile, k * kBatchThreads + tid);
-            stage::geo_entry(mv, g.n, g.ty * g.tx, g.ref, stage::geo_q(g.tile, b.snum, b.sden), b.P.geo,
+            stage::strength(mv, g, b.c.m_th, b.c.s1, b.c.s2, b.P.s_tile, k * kBatchThreads + tid);
+            stage::geo_entry(mv, g, stage::geo_q(g.tile, b.snum, b.sden), b.P.geo,
                              k * kBatchThreads + tid, stage::region_kind(g.tile, b.snum, b.sden) != 0);
             break;
         case S_ROB: {

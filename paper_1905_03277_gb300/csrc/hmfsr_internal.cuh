@@ -162,7 +162,16 @@ struct Geom {
     int n, h, w, pitch, ref, wl;
     int hh, wh;          // half-res size
     int tile, ty, tx;    // motion-field tiles (raw px)
+    // where the frames (and their motion) lie in the caller's burst: in order (src_first < 0), or,
+    // for a chunk of a burst, frame 0 at src_base and frames 1, 2, .. at src_first on, src_base left out
+    int src_base = 0, src_first = -1;
 };
+__host__ __device__ __forceinline__ int src_frame(const Geom &g, int f) {
+    if (g.src_first < 0) return f;
+    if (f == 0) return g.src_base;
+    const int k = g.src_first + f - 1;
+    return k < g.src_base ? k : k + 1;
+}
 
 // Per-frame merge planes in the workspace (one entry per half-res pixel per frame).
 struct MergePlanes {

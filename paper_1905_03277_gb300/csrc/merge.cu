@@ -20,9 +20,9 @@ __global__ void __launch_bounds__(128) k_prep(const uint16_t *__restrict__ burst
                       blockIdx.y * rows, f0 + blockIdx.z, threadIdx.x & 31, rows);
 }
 
-__global__ void k_strength(const float2 *__restrict__ motion, int n, int ty, int tx, float m_th, float s1, float s2,
+__global__ void k_strength(const float2 *__restrict__ motion, Geom g, float m_th, float s1, float s2,
                            float *__restrict__ s_tile) {
-    stage::strength(motion, n, ty, tx, m_th, s1, s2, s_tile, blockIdx.x * blockDim.x + threadIdx.x);
+    stage::strength(motion, g, m_th, s1, s2, s_tile, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // 4 warps side by side: 4 x kRobOut texel columns x `rows` rows of one frame
@@ -44,9 +44,8 @@ __global__ void k_hf_flag(const uint16_t *__restrict__ burst, const uint2 *__res
     stage::hf_flag_px(burst, s1, g, kappa, flag, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y);
 }
 
-__global__ void k_geo(const float2 *__restrict__ motion, int n, int ntl, int ref, int Q, int4 *__restrict__ geo,
-                      bool split) {
-    stage::geo_entry(motion, n, ntl, ref, Q, geo, blockIdx.x * blockDim.x + threadIdx.x, split);
+__global__ void k_geo(const float2 *__restrict__ motion, Geom g, int Q, int4 *__restrict__ geo, bool split) {
+    stage::geo_entry(motion, g, Q, geo, blockIdx.x * blockDim.x + threadIdx.x, split);
 }
 
 template <bool kDen, int SN, int SD>
@@ -264,7 +263,7 @@ cudaError_t launch_merge_prep_motion(const float *motion, const Geom &g, const M
     CheckedLaunches checked(s);
     int nt = g.n * g.ty * g.tx;
     const float2 *mv = reinterpret_cast<const float2 *>(motion);
-    k_strength<<<div_up(nt, 128), 128, 0, s>>>(mv, g.n, g.ty, g.tx, c.m_th, c.s1, c.s2, P.s_tile);
+    k_strength<<<div_up(nt, 128), 128, 0, s>>>(mv, g, c.m_th, c.s1, c.s2, P.s_tile);
     const unsigned char *hf = (c.hf_loss > 0.f && g.n > 1) ? P.hf_flag : nullptr;
     if (g.n > 1) {
         const int slots = hf ? strip_slots(SK_ROB_HF, (const void *)k_rob<true>)
@@ -288,10 +287,9 @@ cudaError_t launch_merge_prep(const uint16_t *burst, const float *motion, const 
 }
 
 cudaError_t launch_geo(const float *motion, const Geom &g, const MergePlanes &P, int snum, int sden, cudaStream_t s) {
-    const int ntl = g.ty * g.tx;
-    k_geo<<<div_up(g.n * ntl, 128), 128, 0, s>>>(reinterpret_cast<const float2 *>(motion), g.n, ntl, g.ref,
-                                                 stage::geo_q(g.tile, snum, sden), P.geo,
-                                                 stage::region_kind(g.tile, snum, sden) != 0);
+    k_geo<<<div_up(g.n * g.ty * g.tx, 128), 128, 0, s>>>(reinterpret_cast<const float2 *>(motion), g,
+                                                         stage::geo_q(g.tile, snum, sden), P.geo,
+                                                         stage::region_kind(g.tile, snum, sden) != 0);
     return cudaGetLastError();
 }
 

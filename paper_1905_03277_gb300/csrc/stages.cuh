@@ -1005,7 +1005,7 @@ __device__ __forceinline__ void prep_strip(const uint16_t *__restrict__ burst, c
                                            uint2 *__restrict__ s1, float4 *__restrict__ base_stats,
                                            float4 *__restrict__ kern, int u0, int v0, int f, int lane,
                                            int rows = kPrepStrip) {
-    const uint16_t *fr = burst + (size_t)f * g.h * g.pitch;
+    const uint16_t *fr = burst + (size_t)src_frame(g, f) * g.h * g.pitch;
     const int u = u0 + lane, uc = min(u, g.wh - 1);
     const bool halo = (lane == 0 || lane == 31);
     const int uh = clampi(lane == 0 ? u0 - 1 : u0 + 32, 0, g.wh - 1);
@@ -1052,11 +1052,13 @@ __device__ __forceinline__ bool motion_span_exceeds(const float2 *__restrict__ m
     return length_exceeds(__dadd_rn(__dmul_rn(Mx, Mx), __dmul_rn(My, My)), m_th);
 }
 
-__device__ __forceinline__ void strength(const float2 *__restrict__ motion, int n, int ty, int tx, float m_th, float s1,
+__device__ __forceinline__ void strength(const float2 *__restrict__ motion, const Geom &g, float m_th, float s1,
                                          float s2, float *__restrict__ s_tile, int i) {
-    if (i >= n * ty * tx) return;
-    int f = i / (ty * tx), r = i % (ty * tx), y = r / tx, x = r % tx;
-    HMFSR_ST(s_tile + i, motion_span_exceeds(motion + (size_t)f * ty * tx, ty, tx, y, x, m_th) ? s1 : s2);
+    const int ntl = g.ty * g.tx;
+    if (i >= g.n * ntl) return;
+    const int f = i / ntl, r = i - f * ntl, y = r / g.tx, x = r - y * g.tx;
+    const float2 *mv = motion + (size_t)src_frame(g, f) * ntl;
+    HMFSR_ST(s_tile + i, motion_span_exceeds(mv, g.ty, g.tx, y, x, m_th) ? s1 : s2);
 }
 
 // --------------------------------------------------------------------------------------
@@ -1070,7 +1072,7 @@ __device__ __forceinline__ void strength(const float2 *__restrict__ motion, int 
 __device__ __forceinline__ void hf_flag_px(const uint16_t *__restrict__ burst, const uint2 *__restrict__ s1,
                                            const Geom &g, float kappa, unsigned char *__restrict__ flag, int u, int v) {
     if (u >= g.wh || v >= g.hh) return;
-    const uint16_t *fr = burst + (size_t)g.ref * g.h * g.pitch;
+    const uint16_t *fr = burst + (size_t)src_frame(g, g.ref) * g.h * g.pitch;
     const uint2 *S = s1 + (size_t)g.ref * g.hh * g.wh;
     long long sq[3] = {0, 0, 0};  // 3x3 sums of squared guide values at (u, v)
     for (int j = -1; j <= 1; ++j)
@@ -1176,7 +1178,7 @@ __device__ __forceinline__ void rob_strip(const uint2 *__restrict__ s1, const fl
     const int txi = min(uc / ht, g.tx - 1);
     const uint2 *S1b = s1 + (size_t)g.ref * hw;
     const uint2 *S1n = s1 + (size_t)frame * hw;
-    const float2 *mvf = motion + (size_t)frame * g.ty * g.tx + txi;
+    const float2 *mvf = motion + (size_t)src_frame(g, frame) * g.ty * g.tx + txi;
     const float *stf = s_tile + (size_t)frame * g.ty * g.tx + txi;
     float *out = rhat + (size_t)frame * hw;
     const int vfirst = max(v0 - 2, 0);
@@ -1206,7 +1208,7 @@ __device__ __forceinline__ void rob_strip(const uint2 *__restrict__ s1, const fl
                 x1 = clampi(uc + (int)flx + 1, 0, wh - 1);
                 x2 = clampi(uc + (int)flx + 2, 0, wh - 1);
                 have_prev = false;
-                if (kHF) span = motion_span_exceeds(motion + (size_t)frame * g.ty * g.tx, g.ty, g.tx, tyi, txi, m_th);
+                if (kHF) span = motion_span_exceeds(mvf - txi, g.ty, g.tx, tyi, txi, m_th);
             }
             if (++tr == ht) { tr = 0; ++tq; }
             const int iy = v + fly;
