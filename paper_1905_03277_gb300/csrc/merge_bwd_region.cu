@@ -508,33 +508,42 @@ __global__ void __launch_bounds__(kRpW *kRpH) k_rpath_region(const float *__rest
     }
 }
 
-// every tile's motion gradient: its regions' and its 8 x 8-texel blocks' sums, in a fixed order
-__global__ void k_motion_region(const float2 *__restrict__ vbar_region, const float2 *__restrict__ vbar_block, Geom g,
-                                int off, int parts, float2 *__restrict__ grad_motion) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= g.n * g.ty * g.tx) return;
-    const int f = t / (g.ty * g.tx), r = t - f * g.ty * g.tx, ty = r / g.tx, tx = r - ty * g.tx;
+// Every tile's motion gradient: its regions' and its 8 x 8-texel blocks' sums, in a fixed order.
+// Eight lanes per tile, so that a tile's loads (up to 16 parts of each region) are in flight
+// together: latency is all of it.  One lane per tile took 23 us for the 256 x 320 x 4 crop at 2x
+// and 17 for 1 MP x 8 at 3/2; this 8 and 18 (FP64 sums).
+constexpr int kTileLanes = 8;
+__global__ void __launch_bounds__(128) k_motion_region(const float2 *__restrict__ vbar_region, const float2 *__restrict__ vbar_block,
+                                                       Geom g, int off, int parts, float2 *__restrict__ grad_motion) {
+    const int t = (blockIdx.x * 128 + threadIdx.x) / kTileLanes, l = threadIdx.x % kTileLanes;
+    const int ntl = g.ty * g.tx, f = t / ntl, r = t - f * ntl, ty = r / g.tx, tx = r - ty * g.tx;
     double x = 0.0, y = 0.0;
-    if (f != g.ref) {
+    if (t < g.n * ntl && f != g.ref) {
         const int nb = g.tile / 16, nbx = div_up(g.wh, 8), nby = div_up(g.hh, 8);
-        const int x0 = tx * nb, x1 = min(x0 + nb, nbx), y0 = ty * nb, y1 = min(y0 + nb, nby);
-        for (int by = y0; by < y1; ++by)
-            for (int bx = x0; bx < x1; ++bx) {
-                const float2 q = vbar_block[((size_t)f * nby + by) * nbx + bx];
-                x += (double)q.x;
-                y += (double)q.y;
-            }
+        const int x0 = tx * nb, y0 = ty * nb, bw = min(x0 + nb, nbx) - x0, bh = min(y0 + nb, nby) - y0;
+        for (int k = l; k < bw * bh; k += kTileLanes) {
+            const int by = k / bw, bx = k - by * bw;
+            const float2 q = __ldg(vbar_block + ((size_t)f * nby + y0 + by) * nbx + x0 + bx);
+            x += (double)q.x;
+            y += (double)q.y;
+        }
         // regions are the same 8 x 8 texels, after `off` leading ones that belong to the first tiles
         const int nrx = nbx + off, nry = nby + off;
-        for (int by = ty == 0 ? 0 : y0 + off; by < y1 + off; ++by)
-            for (int bx = tx == 0 ? 0 : x0 + off; bx < x1 + off; ++bx)
-                for (int k = 0; k < parts; ++k) {  // a warp's sums, each with its rounding error
-                    const float4 q = __ldg(reinterpret_cast<const float4 *>(vbar_region) + (((size_t)f * nry + by) * nrx + bx) * parts + k);
-                    x += (double)q.x + (double)q.y;
-                    y += (double)q.z + (double)q.w;
-                }
+        const int rx0 = tx == 0 ? 0 : x0 + off, ry0 = ty == 0 ? 0 : y0 + off, rw = x0 + bw + off - rx0, rh = y0 + bh + off - ry0;
+        for (int k = l; k < rw * rh * parts; k += kTileLanes) {  // a warp's sums, each with its rounding error
+            const int q0 = k / parts, by = q0 / rw, bx = q0 - by * rw;
+            const float4 q = __ldg(reinterpret_cast<const float4 *>(vbar_region) +
+                                   (((size_t)f * nry + ry0 + by) * nrx + rx0 + bx) * parts + (k - q0 * parts));
+            x += (double)q.x + (double)q.y;
+            y += (double)q.z + (double)q.w;
+        }
     }
-    grad_motion[t] = make_float2((float)x, (float)y);
+#pragma unroll
+    for (int o = kTileLanes / 2; o > 0; o >>= 1) {
+        x += __shfl_xor_sync(0xffffffffu, x, o);
+        y += __shfl_xor_sync(0xffffffffu, y, o);
+    }
+    if (l == 0 && t < g.n * ntl) grad_motion[t] = make_float2((float)x, (float)y);
 }
 
 template <int SN, int SD>
@@ -570,7 +579,7 @@ cudaError_t launch_finish(const Geom &g, const BwdPlanes &B, float *grad_motion,
     constexpr int S = RegionScale<SN, SD>::S, kOff = RegionScale<SN, SD>::kOff;
     k_rpath_region<SN, SD><<<dim3(div_up(g.wh, kRpW), div_up(g.hh, kRpH), g.n), kRpW * kRpH, 0, s>>>(
         B.rhbar_phase, B.flags, B.rb, g, B.vbar_block, B.part2);
-    k_motion_region<<<div_up(g.n * g.ty * g.tx, 64), 64, 0, s>>>(B.vbar_region, B.vbar_block, g, kOff, S * S,
+    k_motion_region<<<div_up(g.n * g.ty * g.tx * kTileLanes, 128), 128, 0, s>>>(B.vbar_region, B.vbar_block, g, kOff, S * S,
                                                                  reinterpret_cast<float2 *>(grad_motion));
     return cudaGetLastError();
 }
