@@ -26,34 +26,6 @@
 namespace hmfsr {
 namespace stage {
 
-// --------------------------------------------------------------------------------------
-// packed FP32 pairs (two IEEE operations per instruction, each rounded as its scalar form)
-// --------------------------------------------------------------------------------------
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-    float2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;"
-        : "=l"(reinterpret_cast<unsigned long long &>(d))
-        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
-          "l"(reinterpret_cast<const unsigned long long &>(c)));
-    return d;
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-    float2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;"
-        : "=l"(reinterpret_cast<unsigned long long &>(d))
-        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)));
-    return d;
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-    float2 d;
-    asm("add.rn.f32x2 %0, %1, %2;"
-        : "=l"(reinterpret_cast<unsigned long long &>(d))
-        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)));
-    return d;
-}
-__device__ __forceinline__ float2 lo2(const float4 &v) { return make_float2(v.x, v.y); }
-__device__ __forceinline__ float2 hi2(const float4 &v) { return make_float2(v.z, v.w); }
-
 struct PairAcc {
     float2 numR, numG, numB, denR, denG, denB, mR, mG, mB;
 };

@@ -176,7 +176,7 @@ __host__ __device__ __forceinline__ int src_frame(const Geom &g, int f) {
 // Per-frame merge planes in the workspace (one entry per half-res pixel per frame).
 struct MergePlanes {
     uint2 *s1;           // [n][hh*wh] 3x3 guide sums {R | B << 16, G1+G2}
-    float4 *base_stats;  // [hh*wh] {max(sum sigma^2, eps), dmd^2 R, G, B} of the base frame
+    float4 *base_stats;  // [hh*wh] {max(sum sigma^2, eps), dmd^2 G, R, B} of the base frame
     float4 *kern;        // [n][hh*wh] kernel covariance as {a, delta, ux, uy}: Omega = a I + delta u u^T
     float *rhat;         // [n][hh*wh] final robustness (base grid); unused for the base frame
     float *s_tile;       // [n][ty*tx] robustness scale from the motion prior

@@ -29,10 +29,10 @@ __global__ void k_strength(const float2 *__restrict__ motion, Geom g, float m_th
 // (blockIdx.z runs over the frames other than the base frame)
 // kHF: with the high-frequency rejection (hf_flag, m_th)
 template <bool kHF>
-__global__ void __launch_bounds__(128) k_rob(const uint2 *__restrict__ s1, const float4 *__restrict__ base_stats,
-                                             const float2 *__restrict__ motion, const float *__restrict__ s_tile,
-                                             Geom g, float t_thr, float *__restrict__ rhat,
-                                             const unsigned char *__restrict__ hf_flag, float m_th, int rows) {
+__global__ void __launch_bounds__(128, 6) k_rob(const uint2 *__restrict__ s1, const float4 *__restrict__ base_stats,
+                                                const float2 *__restrict__ motion, const float *__restrict__ s_tile,
+                                                Geom g, float t_thr, float *__restrict__ rhat,
+                                                const unsigned char *__restrict__ hf_flag, float m_th, int rows) {
     const int frame = (int)blockIdx.z < g.ref ? (int)blockIdx.z : (int)blockIdx.z + 1;
     stage::rob_strip<kHF>(s1, base_stats, motion, s_tile, g, t_thr, rhat,
                           (blockIdx.x * 4 + (threadIdx.x >> 5)) * stage::kRobOut, blockIdx.y * rows, frame,
@@ -269,7 +269,7 @@ cudaError_t launch_merge_prep_motion(const float *motion, const Geom &g, const M
         const int slots = hf ? strip_slots(SK_ROB_HF, (const void *)k_rob<true>)
                              : strip_slots(SK_ROB, (const void *)k_rob<false>);
         const int cols = div_up(g.wh, 4 * stage::kRobOut);
-        const int rows = strip_rows(slots, (long long)cols * (g.n - 1), g.hh, 4, 8, 256, stage::kRobStrip);
+        const int rows = strip_rows(slots, (long long)cols * (g.n - 1), g.hh, 4, 2, 256, stage::kRobStrip);
         const dim3 grid(cols, div_up(g.hh, rows), g.n - 1);
         if (hf)
             k_rob<true><<<grid, 128, 0, s>>>(P.s1, P.base_stats, mv, P.s_tile, g, c.t, P.rhat, hf, c.m_th, rows);

@@ -110,10 +110,10 @@ __global__ void k_rback(const uint2 *__restrict__ s1, const float4 *__restrict__
         float inv, dmd2;
         if (ch == 0) {
             sbv = sb.x & 0xffff; m00 = n00.x & 0xffff; m10 = n10.x & 0xffff; m01 = n01.x & 0xffff; m11 = n11.x & 0xffff;
-            inv = 1.f / 9.f; dmd2 = st.y;
+            inv = 1.f / 9.f; dmd2 = st.z;
         } else if (ch == 1) {
             sbv = sb.y; m00 = n00.y; m10 = n10.y; m01 = n01.y; m11 = n11.y;
-            inv = 1.f / 18.f; dmd2 = st.z;
+            inv = 1.f / 18.f; dmd2 = st.y;
         } else {
             sbv = sb.x >> 16; m00 = n00.x >> 16; m10 = n10.x >> 16; m01 = n01.x >> 16; m11 = n11.x >> 16;
             inv = 1.f / 9.f; dmd2 = st.w;

@@ -12,6 +12,34 @@ namespace stage {
 constexpr float kHalfLog2e = 0.72134752044448170368f;  // log2(e) / 2
 constexpr float kBig = 1.0e30f;
 
+// --------------------------------------------------------------------------------------
+// packed FP32 pairs (two IEEE operations per instruction, each rounded as its scalar form)
+// --------------------------------------------------------------------------------------
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
+          "l"(reinterpret_cast<const unsigned long long &>(c)));
+    return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;"
+        : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)));
+    return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 d;
+    asm("add.rn.f32x2 %0, %1, %2;"
+        : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)));
+    return d;
+}
+__device__ __forceinline__ float2 lo2(const float4 &v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(const float4 &v) { return make_float2(v.z, v.w); }
+
 // ======================================================================================
 // alignment (Sec. 3.2)
 // ======================================================================================
@@ -851,7 +879,7 @@ __device__ __forceinline__ float4 base_stats_of(const uint32_t (&S1)[3], const u
         sig2 += fmaxf(var_ms, var_md);
     }
     float eps = 1e-12f * (float)wl * (float)wl;
-    return make_float4(fmaxf(sig2, eps), dmd2[0], dmd2[1], dmd2[2]);
+    return make_float4(fmaxf(sig2, eps), dmd2[1], dmd2[0], dmd2[2]);
 }
 
 // --------------------------------------------------------------------------------------
@@ -1108,15 +1136,37 @@ __device__ __forceinline__ void hf_flag_px(const uint16_t *__restrict__ burst, c
 
 // --------------------------------------------------------------------------------------
 // robustness (Eq. 5, 6) and its 5x5 minimum (Eq. 9) on one strip of base texels of one
-// frame: one warp, kRobOut columns, `rows` rows.  Each lane evaluates R at two texel
+// frame: one warp, kRobOut columns, `rows` rows (even).  Each lane evaluates R at two texel
 // columns for the rows v0 - 2 .. v0 + rows + 1, walking down: within a motion tile the
 // bilinear neighbours of the row below are the bottom neighbours of this row, so each row
 // reads new sums for the bottom neighbours only.  A rolling window of five row minima
 // gives the column minimum.  Every lane of the warp calls this.
+//
+// Lane l of a warp owns texel columns u0 - 2 + 2 l and u0 - 1 + 2 l (u0 even, so both lie
+// in one motion tile); the warp writes the kRobOut columns u0 .. u0 + kRobOut - 1 (lanes
+// 1 .. 30).  The pair shares the middle column of its bilinear neighbours (three per row),
+// the loop and tile bookkeeping, and a 5-wide row minimum built from the two neighbouring
+// lanes' pairs.
+//
+// A row's latency bounds it: its loads go out together, before the first use of one (each texel's
+// in a branch of its own made three latencies a row), and short strips where the frames leave the
+// chip idle.  More warps than 24 per SM cost time (12 MP x 8 frames: 24 warps 138 us, 32 147, 36
+// 158); packed pairs with a row fetched ahead take 110 registers and more time than they save (150
+// to 190 us), and frames side by side in a block, sharing the base row, 230.  The guide sums stay
+// as the mantissa of 2^23 (exact, and so are the differences of two of them).  At 12 MP x 8 frames
+// 147 us became 138, at 256 x 256 x 8 16 us became 10.
 // --------------------------------------------------------------------------------------
 constexpr int kRobStrip = 64;  // default strip height, as for kPrepStrip
 constexpr float kLog2e = 1.44269504088896340736f;
+constexpr int kRobOut = 60;
 
+struct RobSums {  // guide sums {R, G, B} + 2^23
+    float r, g, b;
+};
+__device__ __forceinline__ RobSums rob_sums(uint2 s) {
+    return {__uint_as_float(__byte_perm(s.x, 0x4B000000u, 0x7610)), __uint_as_float(s.y | 0x4B000000u),
+            __uint_as_float(__byte_perm(s.x, 0x4B000000u, 0x7632))};
+}
 // Wiener-shrunk squared difference of one channel (Eq. 6): (d d^2 / (d^2 + dmd^2))^2 added
 // to dd; a zero denominator means a zero difference
 __device__ __forceinline__ float wiener_add(float d, float dmd2, float dd) {
@@ -1124,42 +1174,19 @@ __device__ __forceinline__ float wiener_add(float d, float dmd2, float dd) {
     const float w = (d * d2) * fast_rcp(fmaxf(d2 + dmd2, 1e-30f));
     return fmaf(w, w, dd);
 }
-
-// --------------------------------------------------------------------------------------
-// Lane l of a warp owns texel columns u0 - 2 + 2 l and u0 - 1 + 2 l (u0 even, so both lie
-// in one motion tile); the warp writes the kRobOut columns u0 .. u0 + kRobOut - 1 (lanes
-// 1 .. 30).  The pair shares the middle column of its bilinear neighbours (three per row),
-// the loop and tile bookkeeping, and a 5-wide row minimum built from the two neighbouring
-// lanes' pairs.  The guide sums become floats exactly (a 16- or 17-bit value in the
-// mantissa of 2^23, minus 2^23), so every difference base - neighbour is exact, as an
-// integer difference would be.
-// --------------------------------------------------------------------------------------
-constexpr int kRobOut = 60;
-
-// exact float of 0 <= v < 2^23
-__device__ __forceinline__ float small_uint_to_float(uint32_t v) { return __uint_as_float(0x4B000000u | v) - 8388608.f; }
-
-struct GuideSums {
-    float r, b, g;
-};
-__device__ __forceinline__ GuideSums guide_sums(uint2 s) {
-    return {small_uint_to_float(s.x & 0xffffu), small_uint_to_float(s.x >> 16), small_uint_to_float(s.y)};
-}
-
 // R of one texel (Eq. 5, 6) from its base sums and the four bilinear neighbours' sums
 // (top-left, top-right, bottom-left, bottom-right) with weights b00 .. b11
-__device__ __forceinline__ float rob_texel(const GuideSums &s, const GuideSums &n00, const GuideSums &n10,
-                                           const GuideSums &n01, const GuideSums &n11, float b00, float b10, float b01,
-                                           float b11, const float4 &st, float sc, float t_thr) {
+__device__ __forceinline__ float rob_texel(const RobSums &s, const RobSums &n00, const RobSums &n10, const RobSums &n01,
+                                           const RobSums &n11, float b00, float b10, float b01, float b11,
+                                           const float4 &st, float sc, float t_thr) {
     float dR = fmaf(b00, s.r - n00.r, fmaf(b10, s.r - n10.r, fmaf(b01, s.r - n01.r, b11 * (s.r - n11.r))));
     float dB = fmaf(b00, s.b - n00.b, fmaf(b10, s.b - n10.b, fmaf(b01, s.b - n01.b, b11 * (s.b - n11.b))));
     float dG = fmaf(b00, s.g - n00.g, fmaf(b10, s.g - n10.g, fmaf(b01, s.g - n01.g, b11 * (s.g - n11.g))));
     dR *= (1.f / 9.f);
     dB *= (1.f / 9.f);
     dG *= (1.f / 18.f);
-    const float dd = wiener_add(dB, st.w, wiener_add(dG, st.z, wiener_add(dR, st.y, 0.f)));
-    const float ex = fast_exp2(-(dd * fast_rcp(st.x)) * kLog2e);
-    return fminf(fmaxf(fmaf(sc, ex, -t_thr), 0.f), 1.f);
+    const float dd = wiener_add(dB, st.w, wiener_add(dG, st.y, wiener_add(dR, st.z, 0.f)));
+    return __saturatef(fmaf(sc, fast_exp2(-(dd * fast_rcp(st.x)) * kLog2e), -t_thr));
 }
 
 // kHF: hf_flag holds the base texels' high-frequency flags, which reject (R = 0) where
@@ -1173,7 +1200,7 @@ __device__ __forceinline__ void rob_strip(const uint2 *__restrict__ s1, const fl
     const size_t hw = (size_t)g.hh * g.wh;
     const int wh = g.wh, ua = u0 - 2 + 2 * lane;
     const bool ok_a = ua >= 0 && ua < wh, ok_b = ua + 1 >= 0 && ua + 1 < wh;
-    const int uc = clampi(ua, 0, wh - 1);
+    const int uc = clampi(ua, 0, wh - 1), db = uc + 1 < wh ? 1 : 0;  // texel b beside a; a where there is none
     const int ht = g.tile / 2;  // motion tile in texels (even)
     const int txi = min(uc / ht, g.tx - 1);
     const uint2 *S1b = s1 + (size_t)g.ref * hw;
@@ -1186,14 +1213,16 @@ __device__ __forceinline__ void rob_strip(const uint2 *__restrict__ s1, const fl
     int cur_tile = -1, fly = 0, x0 = 0, x1 = 0, x2 = 0;
     bool span = false;
     float b00 = 0.f, b10 = 0.f, b01 = 0.f, b11 = 0.f, sc = 0.f;
-    GuideSums t0{}, t1{}, t2{}, n0{}, n1{}, n2{};  // sums at the top / bottom neighbours x0, x1, x2
-    bool have_prev = false;
+    uint2 n0 = make_uint2(0u, 0u), n1 = n0, n2 = n0;  // sums at the bottom neighbours x0, x1, x2
     float ha[4] = {kBig, kBig, kBig, kBig}, hb[4] = {kBig, kBig, kBig, kBig};  // row minima of the rows above
     int off = (v0 - 2) * wh + uc;  // texel a's offset in the row (32-bit offsets)
     for (int e = 0; e < rows + 4; ++e, off += wh) {
         const int v = v0 - 2 + e;
         float ra = kBig, rb = kBig;
         if (v >= 0 && v < g.hh) {  // the same for the whole warp
+            // every load of the row before the first use of one
+            const uint2 sa = HMFSR_LD(S1b + off), sb = HMFSR_LD(S1b + off + db);
+            const float4 pa = HMFSR_LD(base_stats + off), pb = HMFSR_LD(base_stats + off + db);
             const int tyi = min(tq, g.ty - 1);
             if (tyi != cur_tile) {
                 cur_tile = tyi;
@@ -1207,36 +1236,27 @@ __device__ __forceinline__ void rob_strip(const uint2 *__restrict__ s1, const fl
                 x0 = clampi(uc + (int)flx, 0, wh - 1);
                 x1 = clampi(uc + (int)flx + 1, 0, wh - 1);
                 x2 = clampi(uc + (int)flx + 2, 0, wh - 1);
-                have_prev = false;
+                const int o0 = clampi(v + fly, 0, g.hh - 1) * wh;
+                n0 = HMFSR_LD(S1n + o0 + x0);
+                n1 = HMFSR_LD(S1n + o0 + x1);
+                n2 = HMFSR_LD(S1n + o0 + x2);
                 if (kHF) span = motion_span_exceeds(mvf - txi, g.ty, g.tx, tyi, txi, m_th);
             }
             if (++tr == ht) { tr = 0; ++tq; }
-            const int iy = v + fly;
-            if (have_prev) {
-                t0 = n0; t1 = n1; t2 = n2;
-            } else {
-                const int o0 = clampi(iy, 0, g.hh - 1) * wh;
-                t0 = guide_sums(HMFSR_LD(S1n + o0 + x0));
-                t1 = guide_sums(HMFSR_LD(S1n + o0 + x1));
-                t2 = guide_sums(HMFSR_LD(S1n + o0 + x2));
+            const uint2 t0 = n0, t1 = n1, t2 = n2;
+            const int o1 = clampi(v + fly + 1, 0, g.hh - 1) * wh;
+            n0 = HMFSR_LD(S1n + o1 + x0);
+            n1 = HMFSR_LD(S1n + o1 + x1);
+            n2 = HMFSR_LD(S1n + o1 + x2);
+            const RobSums T1 = rob_sums(t1), N1 = rob_sums(n1);
+            ra = rob_texel(rob_sums(sa), rob_sums(t0), T1, rob_sums(n0), N1, b00, b10, b01, b11, pa, sc, t_thr);
+            rb = rob_texel(rob_sums(sb), T1, rob_sums(t2), N1, rob_sums(n2), b00, b10, b01, b11, pb, sc, t_thr);
+            if (kHF) {
+                if (span && HMFSR_LD(hf_flag + off)) ra = 0.f;
+                if (span && HMFSR_LD(hf_flag + off + db)) rb = 0.f;
             }
-            const int o1 = clampi(iy + 1, 0, g.hh - 1) * wh;
-            n0 = guide_sums(HMFSR_LD(S1n + o1 + x0));
-            n1 = guide_sums(HMFSR_LD(S1n + o1 + x1));
-            n2 = guide_sums(HMFSR_LD(S1n + o1 + x2));
-            have_prev = true;
-            if (ok_a) {
-                if (kHF && span && HMFSR_LD(hf_flag + off)) ra = 0.f;
-                else ra = rob_texel(guide_sums(HMFSR_LD(S1b + off)), t0, t1, n0, n1, b00, b10, b01, b11,
-                                    HMFSR_LD(base_stats + off), sc, t_thr);
-            }
-            if (ok_b) {
-                if (kHF && span && HMFSR_LD(hf_flag + off + 1)) rb = 0.f;
-                else rb = rob_texel(guide_sums(HMFSR_LD(S1b + off + 1)), t1, t2, n1, n2, b00, b10, b01, b11,
-                                    HMFSR_LD(base_stats + off + 1), sc, t_thr);
-            }
-        } else {
-            have_prev = false;
+            ra = ok_a ? ra : kBig;
+            rb = ok_b ? rb : kBig;
         }
         // 5-wide row minima: the previous lane's pair, this pair, the next lane's pair
         const float pa = __shfl_up_sync(0xffffffffu, ra, 1), pb = __shfl_up_sync(0xffffffffu, rb, 1);
