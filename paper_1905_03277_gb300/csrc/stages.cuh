@@ -465,8 +465,11 @@ __device__ __forceinline__ void ssd_group(const uint16_t *__restrict__ img, int 
     }
 }
 
-// Lucas-Kanade refinement (Sec. 3.2) of one level-0 tile per warp, on I = Lq / 4.  Each
-// lane owns pixels lane + 32 m of the tile.  Gradients of the base frame by central
+// Lucas-Kanade refinement (Sec. 3.2) of one level-0 tile per warp (T = 16, 32), on I = Lq / 4.
+// A lane owns a run of T T / 32 pixels down one column, so that the gradient rows and the sampled
+// rows roll down the run: two loads and one horizontal interpolation per row and iteration, where
+// pixels taken 32 apart need four and two (loads from L1 bound it: 3 MP x 13 frames, T = 16,
+// 81 us, now 56).  Gradients of the base frame by central
 // differences around the clamped pixel; H = sum g g^T is summed exactly in integers, so
 // the conditioning guard (tr H == 0 or det H <= 1e-9 tr(H)^2) is an exact 128-bit integer
 // test; each iteration accumulates sum g r in FP32 (warp shuffles) and solves the 2x2
@@ -475,7 +478,8 @@ template <int T>
 __device__ __forceinline__ void lk(const uint16_t *__restrict__ L0, int lh, int lw, int lty, int ltx,
                                    const int2 *__restrict__ vec0, int ref, int iters, float *__restrict__ motion,
                                    int32_t *__restrict__ motion_int, int warp, int lane, int f) {
-    constexpr int t = T, npx = T * T, nper = (npx + 31) / 32;
+    static_assert(T == 16 || T == 32, "whole runs");
+    constexpr int kRun = T * T / 32;  // even
     if (warp >= lty * ltx) return;
     const int ty = warp / ltx, tx = warp % ltx;
     const size_t o = (size_t)f * lty * ltx + warp;
@@ -490,21 +494,41 @@ __device__ __forceinline__ void lk(const uint16_t *__restrict__ L0, int lh, int 
     const uint16_t *R = L0 + (size_t)ref * lh * lw;
     const uint16_t *A = L0 + (size_t)f * lh * lw;
     const int2 u = HMFSR_LD(vec0 + o);
-    int gxs[nper], gys[nper], pxs[nper], pys[nper], rv[nper];
+    const int x = min(tx * T + lane % T, lw - 1), xm = max(x - 1, 0), xp = min(x + 1, lw - 1);
+    const int yt = ty * T, y0 = yt + lane / T * kRun;
+    const bool whole = yt + T <= lh;  // no row of the tile is clamped
+    float gxs[kRun], gys[kRun], rv[kRun];
     long long hxx = 0, hxy = 0, hyy = 0;
+    {
+        int pm = 0, c = 0;
+        if (whole) {
+            pm = HMFSR_LDG(R + max(y0 - 1, 0) * lw + x);
+            c = HMFSR_LDG(R + y0 * lw + x);
+        }
+        int gx_even = 0, gy_even = 0;
 #pragma unroll
-    for (int m = 0; m < nper; ++m) {
-        const int k = lane + 32 * m;
-        if (k >= npx) { gxs[m] = gys[m] = 0; pxs[m] = pys[m] = 0; rv[m] = 0; continue; }
-        const int x = min(tx * t + k % t, lw - 1), y = min(ty * t + k / t, lh - 1);
-        const uint16_t *row = R + (size_t)y * lw;
-        const int gx = (int)HMFSR_LDG(row + min(x + 1, lw - 1)) - (int)HMFSR_LDG(row + max(x - 1, 0));
-        const int gy = (int)HMFSR_LDG(R + (size_t)min(y + 1, lh - 1) * lw + x) - (int)HMFSR_LDG(R + (size_t)max(y - 1, 0) * lw + x);
-        gxs[m] = gx; gys[m] = gy; pxs[m] = x; pys[m] = y;
-        rv[m] = HMFSR_LDG(row + x);
-        hxx += (long long)(gx * gx);
-        hxy += (long long)(gx * gy);
-        hyy += (long long)(gy * gy);
+        for (int j = 0; j < kRun; ++j) {
+            const int y = min(y0 + j, lh - 1);
+            const uint16_t *row = R + y * lw;  // 32-bit offsets: a level holds < 2^31 texels
+            if (!whole) {
+                pm = HMFSR_LDG(R + max(y - 1, 0) * lw + x);
+                c = HMFSR_LDG(row + x);
+            }
+            const int n = HMFSR_LDG(R + min(y + 1, lh - 1) * lw + x);
+            const int gx = (int)HMFSR_LDG(row + xp) - (int)HMFSR_LDG(row + xm), gy = n - pm;
+            gxs[j] = (float)gx * 0.125f;
+            gys[j] = (float)gy * 0.125f;
+            rv[j] = (float)c;
+            if (j & 1) {  // |g| < 2^15: two squares or products fit a 32-bit int
+                hxx += (long long)(gx_even * gx_even + gx * gx);
+                hxy += (long long)(gx_even * gy_even + gx * gy);
+                hyy += (long long)(gy_even * gy_even + gy * gy);
+            }
+            gx_even = gx;
+            gy_even = gy;
+            pm = c;
+            c = n;
+        }
     }
     hxx = warp_sum_ll(hxx);
     hxy = warp_sum_ll(hxy);
@@ -522,20 +546,34 @@ __device__ __forceinline__ void lk(const uint16_t *__restrict__ L0, int lh, int 
             const float fdx = floorf(dx), fdy = floorf(dy);
             const float ax = dx - fdx, ay = dy - fdy;
             const int ox = u.x + (int)fdx, oy = u.y + (int)fdy;
+            const int s0 = clampi(x + ox, 0, lw - 1), s1 = clampi(x + ox + 1, 0, lw - 1);
             float bx = 0.f, by = 0.f;
-#pragma unroll
-            for (int m = 0; m < nper; ++m) {
-                if (lane + 32 * m >= npx) continue;
-                const int ix = pxs[m] + ox, iy = pys[m] + oy;
-                const int x0 = clampi(ix, 0, lw - 1), x1 = clampi(ix + 1, 0, lw - 1);
-                const uint16_t *a0 = A + (size_t)clampi(iy, 0, lh - 1) * lw;
-                const uint16_t *a1 = A + (size_t)clampi(iy + 1, 0, lh - 1) * lw;
-                const float i00 = HMFSR_LDG(a0 + x0), i10 = HMFSR_LDG(a0 + x1), i01 = HMFSR_LDG(a1 + x0), i11 = HMFSR_LDG(a1 + x1);
-                const float top = fmaf(ax, i10, (1.f - ax) * i00), bot = fmaf(ax, i11, (1.f - ax) * i01);
+            auto row_at = [&](const uint16_t *a) {
+                return fmaf(ax, (float)HMFSR_LDG(a + s1), (1.f - ax) * (float)HMFSR_LDG(a + s0));
+            };
+            auto add = [&](int j, float top, float bot) {
                 const float ia = fmaf(ay, bot, (1.f - ay) * top);
-                const float r = (ia - (float)rv[m]) * 0.25f;
-                bx = fmaf((float)gxs[m] * 0.125f, r, bx);
-                by = fmaf((float)gys[m] * 0.125f, r, by);
+                const float r = (ia - rv[j]) * 0.25f;
+                bx = fmaf(gxs[j], r, bx);
+                by = fmaf(gys[j], r, by);
+            };
+            if (whole && yt + oy >= 0 && yt + oy + T < lh) {
+                // the tile's rows and the sampled rows are inside the level: one row after another
+                const uint16_t *a = A + (y0 + oy) * lw;
+                float top = row_at(a);
+#pragma unroll
+                for (int j = 0; j < kRun; ++j) {
+                    a += lw;
+                    const float bot = row_at(a);
+                    add(j, top, bot);
+                    top = bot;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < kRun; ++j) {
+                    const int iy = min(y0 + j, lh - 1) + oy;
+                    add(j, row_at(A + clampi(iy, 0, lh - 1) * lw), row_at(A + clampi(iy + 1, 0, lh - 1) * lw));
+                }
             }
             bx = warp_sum_f(bx);
             by = warp_sum_f(by);
