@@ -108,23 +108,36 @@ __global__ void __launch_bounds__(128) k_ssd_group(const uint16_t *__restrict__ 
 // (as ints, each row once, through 16-byte loads where the rows allow); every lane then
 // reads its rows from there with 16-byte shared loads.  Same sums and keys as ssd_group,
 // so the same vectors.
+//
+// Bounded by the integer multiplier (it issues every other cycle, and takes plain
+// subtractions too).  Where whole rows fit a 32-bit partial (PART >= T) the square is
+// therefore expanded: sum (r - a)^2 = sum r^2 + sum a^2 - 2 sum r a, one multiply-add a term,
+// with sum a^2 of each row's windows made once by the lane that stages the row.  The three sums
+// are taken modulo 2^32, where a partial of (r - a)^2 terms is exact because it fits.  The
+// shared-memory path is then the bound (90 %).  Level 1 of 12 MP x 8 frames, T = 8: radius 4 70 us
+// with r - a squared, 60 so; the whole alignment at radius 7 347 us and 314.  T = 16, radius 4, 3 MP
+// x 13: 60 us in k_ssd_tile, 27 here.
 template <int T, int RAD>
 struct StagedSsd {
     static constexpr int kW = 2 * RAD + 1, kG = 32 / kW, kA = T + 2 * RAD;
     static constexpr int kS = ((kA + 3) & ~3) + 4;  // window row stride (ints): 16-byte rows, banks spread
+    static constexpr int kQ = ((kW + 3) & ~3) | 4;  // sums of squares of a row's windows; 4 mod 8, so that 8 rows share no bank
     static constexpr int kWin = kA * kS;
-    static constexpr int kTile = kWin + T * T;      // ints per tile: window, then the T x T reference
-    static constexpr int kWarps = 4;
+    static constexpr int kRef = kWin, kSq = kWin + T * T, kSr = kSq + kA * kQ;
+    static constexpr int kTile = kSr + ((T + 3) & ~3);  // ints per tile: window, T x T reference, sums of squares
+    static constexpr int kWarps = T <= 8 ? 4 : (RAD >= 3 ? 2 : 1);
+    static constexpr bool kExpand = T >= 8 || RAD >= 5;  // too few terms otherwise (12 MP, T = 4: 363 us against 351)
     static constexpr size_t kBytes = sizeof(int) * kWarps * kG * kTile;
 };
 
 template <int T, int RAD, int PART>
-__global__ void __launch_bounds__(128) k_ssd_staged(const uint16_t *__restrict__ img, int lh, int lw, int lty, int ltx,
-                                                    const int2 *__restrict__ parent, int pty, int ptx, int fsh,
-                                                    int ref, int2 *__restrict__ vec) {
+__global__ void __launch_bounds__(32 * StagedSsd<T, RAD>::kWarps)
+    k_ssd_staged(const uint16_t *__restrict__ img, int lh, int lw, int lty, int ltx, const int2 *__restrict__ parent, int pty,
+                 int ptx, int fsh, int ref, int2 *__restrict__ vec) {
     using S = StagedSsd<T, RAD>;
-    constexpr int kW = S::kW, kG = S::kG, kA = S::kA, kS = S::kS;
-    static_assert(T % 4 == 0 && kS % 4 == 0, "16-byte shared rows");
+    constexpr int kW = S::kW, kG = S::kG, kA = S::kA, kS = S::kS, kQ = S::kQ;
+    constexpr bool kExpand = S::kExpand && PART >= T;
+    static_assert(T % 4 == 0 && kS % 4 == 0 && S::kTile % 4 == 0 && S::kSq % 4 == 0 && kQ % 4 == 0, "16-byte shared rows");
     __shared__ __align__(16) int sm[S::kWarps][kG][S::kTile];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, f = blockIdx.y;
     const int tile0 = (blockIdx.x * S::kWarps + warp) * kG, ntiles = lty * ltx;
@@ -155,8 +168,23 @@ __global__ void __launch_bounds__(128) k_ssd_staged(const uint16_t *__restrict__
 #pragma unroll
             for (int i = kA & ~3; i < kA; ++i) sm[warp][g][rr * kS + i] = v[i];
         }
+        if constexpr (kExpand) {
+            int q[(kW + 3) & ~3] = {};  // modulo 2^32
+            unsigned int sum = 0;
+#pragma unroll
+            for (int i = 0; i < T; ++i) sum += (unsigned int)v[i] * (unsigned int)v[i];
+            q[0] = (int)sum;
+#pragma unroll
+            for (int k = 1; k < kW; ++k) {
+                sum += (unsigned int)v[k + T - 1] * (unsigned int)v[k + T - 1] - (unsigned int)v[k - 1] * (unsigned int)v[k - 1];
+                q[k] = (int)sum;
+            }
+            int4 *dq = reinterpret_cast<int4 *>(&sm[warp][g][S::kSq + rr * kQ]);
+#pragma unroll
+            for (int i = 0; i < (kW + 3) / 4; ++i) dq[i] = make_int4(q[4 * i], q[4 * i + 1], q[4 * i + 2], q[4 * i + 3]);
+        }
     }
-    // reference rows: kG x T rows
+    // reference rows: kG x T rows; expanded, as -2 r beside the row's sum of squares
     for (int r = lane; r < kG * T; r += 32) {
         const int g = r / T, j = r - g * T, t = tile0 + g;
         if (t >= ntiles) continue;
@@ -165,7 +193,16 @@ __global__ void __launch_bounds__(128) k_ssd_staged(const uint16_t *__restrict__
         const bool inside = x0 + T <= lw;
         int v[T];
         stage::load_row2<T, T % 8 == 0>(R + (size_t)min(y0 + j, lh - 1) * lw, x0, lw, inside, inside && al16, v);
-        int4 *dst = reinterpret_cast<int4 *>(&sm[warp][g][S::kWin + j * T]);
+        if constexpr (kExpand) {
+            unsigned int q = 0;
+#pragma unroll
+            for (int i = 0; i < T; ++i) {
+                q += (unsigned int)v[i] * (unsigned int)v[i];
+                v[i] *= -2;
+            }
+            sm[warp][g][S::kSr + j] = (int)q;
+        }
+        int4 *dst = reinterpret_cast<int4 *>(&sm[warp][g][S::kRef + j * T]);
 #pragma unroll
         for (int i = 0; i < T / 4; ++i) dst[i] = make_int4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
     }
@@ -173,11 +210,8 @@ __global__ void __launch_bounds__(128) k_ssd_staged(const uint16_t *__restrict__
     unsigned long long best = ~0ull;
     if (active) {
         const int *win = &sm[warp][grp][d * kS];  // candidate row j + d of the window at row j
-        const int *rf = &sm[warp][grp][S::kWin];
-        stage::SsdAcc<T, PART> acc[kW];
-#pragma unroll 2
-        for (int j = 0; j < T; ++j) {
-            int rv[T], av[kA];
+        const int *rf = &sm[warp][grp][S::kRef];
+        auto load_rows = [&](int j, int (&rv)[T], int (&av)[kA]) {
             const int4 *pr = reinterpret_cast<const int4 *>(rf + j * T);
             const int4 *pa = reinterpret_cast<const int4 *>(win + j * kS);
 #pragma unroll
@@ -194,13 +228,59 @@ __global__ void __launch_bounds__(128) k_ssd_staged(const uint16_t *__restrict__
 #pragma unroll
                 for (int i = kA & ~3; i < kA; ++i) av[i] = win[j * kS + i];
             }
+        };
+        if constexpr (kExpand) {
+            constexpr int kRows = PART / T;  // rows per 32-bit partial
+            const int *sq = &sm[warp][grp][S::kSq + d * kQ], *sr = &sm[warp][grp][S::kSr];
+            unsigned long long total[kW];
 #pragma unroll
-            for (int k = 0; k < kW; ++k) acc[k].add(rv, av + k, j);
-        }
+            for (int k = 0; k < kW; ++k) total[k] = 0ull;
+#pragma unroll 1
+            for (int j0 = 0; j0 < T; j0 += kRows) {
+                unsigned int part[kW];
 #pragma unroll
-        for (int k = 0; k < kW; ++k) {
-            const unsigned long long key = stage::ssd_key(acc[k].total, k - RAD, d - RAD);
-            best = key < best ? key : best;
+                for (int jj = 0; jj < kRows && jj < T; ++jj) {
+                    const int j = j0 + jj;
+                    if (T % kRows != 0 && j >= T) break;
+                    int rv[T], av[kA];
+                    load_rows(j, rv, av);
+                    const unsigned int s = (unsigned int)sr[j];
+                    int q[(kW + 3) & ~3];
+#pragma unroll
+                    for (int i = 0; i < (kW + 3) / 4; ++i) {
+                        const int4 w = reinterpret_cast<const int4 *>(sq + j * kQ)[i];
+                        q[4 * i] = w.x; q[4 * i + 1] = w.y; q[4 * i + 2] = w.z; q[4 * i + 3] = w.w;
+                    }
+#pragma unroll
+                    for (int k = 0; k < kW; ++k) {
+                        unsigned int p = (unsigned int)q[k] + s + (jj ? part[k] : 0u);
+#pragma unroll
+                        for (int i = 0; i < T; ++i) p += (unsigned int)rv[i] * (unsigned int)av[k + i];
+                        part[k] = p;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < kW; ++k) total[k] += part[k];
+            }
+#pragma unroll
+            for (int k = 0; k < kW; ++k) {
+                const unsigned long long key = stage::ssd_key(total[k], k - RAD, d - RAD);
+                best = key < best ? key : best;
+            }
+        } else {
+            stage::SsdAcc<T, PART> acc[kW];
+#pragma unroll 2
+            for (int j = 0; j < T; ++j) {
+                int rv[T], av[kA];
+                load_rows(j, rv, av);
+#pragma unroll
+                for (int k = 0; k < kW; ++k) acc[k].add(rv, av + k, j);
+            }
+#pragma unroll
+            for (int k = 0; k < kW; ++k) {
+                const unsigned long long key = stage::ssd_key(acc[k].total, k - RAD, d - RAD);
+                best = key < best ? key : best;
+            }
         }
     }
     // idle lanes read the last group (their result is unused)
@@ -275,23 +355,27 @@ __global__ void k_lk(const uint16_t *__restrict__ L0, int lh, int lw, int lty, i
 // dy spread over the lanes of a group (measured at 12 MP on level 1, 96k tile-frames: the
 // grouped form 9 us faster than one thread per tile, both at 64 registers).
 
-// at most this many tile-frames: a level is searched one tile per block (k_ssd_tile)
-constexpr long long kTileSearchMax = 16384;
+// at most this many tile-frames (of T x T texels): a level is searched one tile per block
+// (k_ssd_tile), which takes the latency of one candidate's sum but reads shared memory twice a term
+// (T = 16, radius 4: 624 tile-frames 10 us, 9984 60 us against 27 staged).  With radius 1 and T = 16
+// the staged windows are mostly halo, and k_ssd_group takes 36 us where they take 50.
+template <int T>
+constexpr long long kTileSearchMax = T <= 8 ? 16384 : 4096;
 
 template <int T, int RAD, int PART>
 static void launch_ssd_part(const AlignLevels &L, int l, int n, int ref, int fsh, bool top, cudaStream_t s) {
     const int tiles = L.lty[l] * L.ltx[l];
     const int2 *parent = top ? nullptr : L.vec[l + 1];
     const int pty = top ? 0 : L.lty[l + 1], ptx = top ? 0 : L.ltx[l + 1];
-    if (RAD >= 2 && (long long)tiles * n <= kTileSearchMax) {
+    if (RAD >= 2 && (long long)tiles * n <= kTileSearchMax<T>) {
         k_ssd_tile<T, RAD, PART><<<dim3(tiles, n), TileSsd<T, RAD>::kThreads, 0, s>>>(
             L.img[l], L.lh[l], L.lw[l], L.lty[l], L.ltx[l], parent, pty, ptx, fsh, ref, L.vec[l]);
     } else if constexpr (RAD <= 2 && T <= 8) {
         k_ssd_rows<T, RAD, PART><<<dim3(div_up(tiles, 64), n), 64, 0, s>>>(
             L.img[l], L.lh[l], L.lw[l], L.lty[l], L.ltx[l], parent, pty, ptx, fsh, ref, L.vec[l]);
-    } else if constexpr (T <= 16 && StagedSsd<T, RAD>::kBytes <= 40 * 1024) {
+    } else if constexpr (T <= 16 && (T <= 8 || RAD >= 2) && StagedSsd<T, RAD>::kBytes <= 44 * 1024) {
         constexpr int kTilesPerBlock = StagedSsd<T, RAD>::kWarps * StagedSsd<T, RAD>::kG;
-        k_ssd_staged<T, RAD, PART><<<dim3(div_up(tiles, kTilesPerBlock), n), 128, 0, s>>>(
+        k_ssd_staged<T, RAD, PART><<<dim3(div_up(tiles, kTilesPerBlock), n), 32 * StagedSsd<T, RAD>::kWarps, 0, s>>>(
             L.img[l], L.lh[l], L.lw[l], L.lty[l], L.ltx[l], parent, pty, ptx, fsh, ref, L.vec[l]);
     } else {
         constexpr int kTilesPerBlock = 4 * (32 / (2 * RAD + 1));
