@@ -336,9 +336,9 @@ hmfsr_status hmfsr_merge(const uint16_t *burst_dev, const hmfsr_burst_desc *desc
     chk.add(rgb_dev, rgb_bytes(desc, scale_num, scale_den));
     chk.add(den_dev, rgb_bytes(desc, scale_num, scale_den));
     chk.add_ws(ws, need);
-    cudaError_t e = launch_merge_prep(burst_dev, motion_dev, g, c, P, s);
+    cudaError_t e = launch_merge_prep(burst_dev, motion_dev, g, c, P, s, scale_num, scale_den);
     if (e != cudaSuccess) return HMFSR_ERR_CUDA;
-    return cuda_status(launch_merge_accum(burst_dev, motion_dev, g, P, scale_num, scale_den, rgb_dev, den_dev, s));
+    return cuda_status(launch_merge_accum(burst_dev, motion_dev, g, P, scale_num, scale_den, rgb_dev, den_dev, true, s));
 }
 
 hmfsr_status hmfsr_align_merge(const uint16_t *burst_dev, const hmfsr_burst_desc *desc,
@@ -381,8 +381,8 @@ hmfsr_status hmfsr_align_merge(const uint16_t *burst_dev, const hmfsr_burst_desc
     const cudaError_t ef = launch_merge_prep_frames(burst_dev, g, c, P, s);
     const cudaError_t ew = cudaStreamWaitEvent(s, side->join, 0);
     if (ea != cudaSuccess || ej != cudaSuccess || ef != cudaSuccess || ew != cudaSuccess) return HMFSR_ERR_CUDA;
-    if (launch_merge_prep_motion(motion_dev, g, c, P, s) != cudaSuccess) return HMFSR_ERR_CUDA;
-    return cuda_status(launch_merge_accum(burst_dev, motion_dev, g, P, scale_num, scale_den, rgb_dev, den_dev, s));
+    if (launch_merge_prep_motion(motion_dev, g, c, P, s, scale_num, scale_den) != cudaSuccess) return HMFSR_ERR_CUDA;
+    return cuda_status(launch_merge_accum(burst_dev, motion_dev, g, P, scale_num, scale_den, rgb_dev, den_dev, true, s));
 }
 
 size_t hmfsr_merge_chunked_workspace_size(const hmfsr_burst_desc *desc, int tile, int scale_num, int scale_den,
@@ -427,10 +427,10 @@ hmfsr_status hmfsr_merge_chunked(const uint16_t *burst_dev, const hmfsr_burst_de
         gc.src_first = o0;
         // the base frame's planes (slot 0) are made by the first chunk and kept
         if (launch_merge_prep_frames(burst_dev, gc, c, L.P, s, ci > 0 ? 1 : 0) != cudaSuccess ||
-            launch_merge_prep_motion(motion_dev, gc, c, L.P, s) != cudaSuccess)
+            launch_merge_prep_motion(motion_dev, gc, c, L.P, s, scale_num, scale_den) != cudaSuccess)
             return HMFSR_ERR_CUDA;
         const bool last = (ci == chunks - 1);
-        if (launch_merge_accum_chunk(burst_dev, motion_dev, gc, L.P, scale_num, scale_den, rgb_dev, den_dev,
+        if (launch_merge_accum_chunk(burst_dev, gc, L.P, scale_num, scale_den, rgb_dev, den_dev,
                                      ci > 0 ? L.state : nullptr, last ? nullptr : L.state, ci > 0, s) != cudaSuccess)
             return HMFSR_ERR_CUDA;
     }
@@ -463,9 +463,9 @@ hmfsr_status hmfsr_merge_noise(const uint16_t *burst_dev, const hmfsr_burst_desc
     chk.add(den_dev, rgb_bytes(desc, scale_num, scale_den));
     chk.add(noise_table_dev, sizeof(float4) * kNoiseLevels);
     chk.add_ws(ws, need);
-    cudaError_t e = launch_merge_prep(burst_dev, motion_dev, g, c, P, s);
+    cudaError_t e = launch_merge_prep(burst_dev, motion_dev, g, c, P, s, scale_num, scale_den);
     if (e != cudaSuccess) return HMFSR_ERR_CUDA;
-    return cuda_status(launch_merge_accum(burst_dev, motion_dev, g, P, scale_num, scale_den, rgb_dev, den_dev, s));
+    return cuda_status(launch_merge_accum(burst_dev, motion_dev, g, P, scale_num, scale_den, rgb_dev, den_dev, true, s));
 }
 
 hmfsr_status hmfsr_merge_ex(const uint16_t *burst_dev, const hmfsr_burst_desc *desc, const float *motion_dev,
@@ -495,9 +495,9 @@ hmfsr_status hmfsr_merge_ex(const uint16_t *burst_dev, const hmfsr_burst_desc *d
     chk.add(den_dev, rgb_bytes(desc, scale_num, scale_den));
     chk.add(opts->noise_table, sizeof(float4) * kNoiseLevels);
     chk.add_ws(ws, need);
-    cudaError_t e = launch_merge_prep(burst_dev, motion_dev, g, c, P, s);
+    cudaError_t e = launch_merge_prep(burst_dev, motion_dev, g, c, P, s, scale_num, scale_den);
     if (e != cudaSuccess) return HMFSR_ERR_CUDA;
-    return cuda_status(launch_merge_accum(burst_dev, motion_dev, g, P, scale_num, scale_den, rgb_dev, den_dev, s));
+    return cuda_status(launch_merge_accum(burst_dev, motion_dev, g, P, scale_num, scale_den, rgb_dev, den_dev, true, s));
 }
 
 hmfsr_status hmfsr_merge_prepare(const uint16_t *burst_dev, const hmfsr_burst_desc *desc, const float *motion_dev,
@@ -539,7 +539,8 @@ hmfsr_status hmfsr_merge_accumulate(const uint16_t *burst_dev, const hmfsr_burst
     chk.add(den_dev, rgb_bytes(desc, scale_num, scale_den));
     chk.add_ws(ws, need);
     return cuda_status(
-        launch_merge_accum(burst_dev, motion_dev, g, P, scale_num, scale_den, rgb_dev, den_dev, (cudaStream_t)stream));
+        launch_merge_accum(burst_dev, motion_dev, g, P, scale_num, scale_den, rgb_dev, den_dev, false,
+                           (cudaStream_t)stream));
 }
 
 hmfsr_status hmfsr_merge_stages(const uint16_t *burst_dev, const hmfsr_burst_desc *desc, const float *motion_dev,

@@ -624,8 +624,8 @@ hmfsr_status hmfsr_batch_run(hmfsr_batch_plan plan, const uint16_t *const *burst
                     const BatchBurst &bb = plan->host[b];
                     cudaStream_t bs = br[r % ns];
                     launch_align(bb.burst, bb.g, plan->ap[b], bb.L, bb.motion, nullptr, bs);
-                    launch_merge_prep(bb.burst, bb.motion, bb.g, bb.c, bb.P, bs);
-                    launch_merge_accum(bb.burst, bb.motion, bb.g, bb.P, bb.snum, bb.sden, bb.rgb, nullptr, bs);
+                    launch_merge_prep(bb.burst, bb.motion, bb.g, bb.c, bb.P, bs, bb.snum, bb.sden);
+                    launch_merge_accum(bb.burst, bb.motion, bb.g, bb.P, bb.snum, bb.sden, bb.rgb, nullptr, true, bs);
                 }
                 for (int i = 0; i < ns; ++i) {
                     cudaEventRecord(ev[i], br[i]);

@@ -223,20 +223,21 @@ cudaError_t launch_align_quadfit(const uint16_t *burst, const Geom &g, const hmf
 
 // merge; launch_merge_prep == launch_merge_prep_frames (the motion-free part: 3x3 sums,
 // base statistics, kernel covariances, high-frequency flags) + launch_merge_prep_motion
-// (motion strength and robustness)
+// (motion strength and robustness; with snum > 0 also launch_geo's table for that output scale)
 cudaError_t launch_merge_prep(const uint16_t *burst, const float *motion, const Geom &g, const MergeConsts &c,
-                              const MergePlanes &P, cudaStream_t s);
+                              const MergePlanes &P, cudaStream_t s, int snum = 0, int sden = 1);
 // first_frame: frames first_frame .. n - 1 only (the planes of the earlier ones are kept)
 cudaError_t launch_merge_prep_frames(const uint16_t *burst, const Geom &g, const MergeConsts &c, const MergePlanes &P,
                                      cudaStream_t s, int first_frame = 0);
 cudaError_t launch_merge_prep_motion(const float *motion, const Geom &g, const MergeConsts &c, const MergePlanes &P,
-                                     cudaStream_t s);
+                                     cudaStream_t s, int snum = 0, int sden = 1);
+// have_geo: the preparation wrote P.geo for this scale
 cudaError_t launch_merge_accum(const uint16_t *burst, const float *motion, const Geom &g, const MergePlanes &P,
-                               int snum, int sden, float *rgb, float *den, cudaStream_t s);
+                               int snum, int sden, float *rgb, float *den, bool have_geo, cudaStream_t s);
 // the accumulation of one chunk of frames of a bounded-memory merge: the running sums
 // from state_in (nullptr: start empty) to state_out (nullptr: normalise into rgb / den);
-// skip_base: the chunk's burst holds the base frame for the statistics only
-cudaError_t launch_merge_accum_chunk(const uint16_t *burst, const float *motion, const Geom &g, const MergePlanes &P,
+// skip_base: the chunk holds the base frame for the statistics only.  P.geo is prepared.
+cudaError_t launch_merge_accum_chunk(const uint16_t *burst, const Geom &g, const MergePlanes &P,
                                      int snum, int sden, float *rgb, float *den, const float *state_in,
                                      float *state_out, bool skip_base, cudaStream_t s);
 // the window geometry of every (frame, tile) for an output scale, into P.geo

@@ -48,6 +48,16 @@ __global__ void k_geo(const float2 *__restrict__ motion, Geom g, int Q, int4 *__
     stage::geo_entry(motion, g, Q, geo, blockIdx.x * blockDim.x + threadIdx.x, split);
 }
 
+// k_strength and k_geo in one launch, where the scale is known before the robustness.  12 MP x 8
+// frames: 18 + 4.4 us apart, with branches around the neighbours beyond the border and FP64 for
+// every tile; 6 so.
+__global__ void k_tiles(const float2 *__restrict__ motion, Geom g, float m_th, float s1, float s2,
+                        float *__restrict__ s_tile, int Q, int4 *__restrict__ geo, bool split) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    stage::strength(motion, g, m_th, s1, s2, s_tile, i);
+    stage::geo_entry(motion, g, Q, geo, i, split);
+}
+
 template <bool kDen, int SN, int SD>
 __global__ void __launch_bounds__(kMergeW *kMergeH, 8) k_merge(const uint16_t *__restrict__ burst,
                                                            const int4 *__restrict__ geo, Geom g,
@@ -258,12 +268,16 @@ cudaError_t launch_merge_prep_frames(const uint16_t *burst, const Geom &g, const
 }
 
 cudaError_t launch_merge_prep_motion(const float *motion, const Geom &g, const MergeConsts &c, const MergePlanes &P,
-                                     cudaStream_t s) {
+                                     cudaStream_t s, int snum, int sden) {
     StageRange range("hmfsr merge: robustness");
     CheckedLaunches checked(s);
     int nt = g.n * g.ty * g.tx;
     const float2 *mv = reinterpret_cast<const float2 *>(motion);
-    k_strength<<<div_up(nt, 128), 128, 0, s>>>(mv, g, c.m_th, c.s1, c.s2, P.s_tile);
+    if (snum > 0)
+        k_tiles<<<div_up(nt, 128), 128, 0, s>>>(mv, g, c.m_th, c.s1, c.s2, P.s_tile, stage::geo_q(g.tile, snum, sden),
+                                                P.geo, stage::region_kind(g.tile, snum, sden) != 0);
+    else
+        k_strength<<<div_up(nt, 128), 128, 0, s>>>(mv, g, c.m_th, c.s1, c.s2, P.s_tile);
     const unsigned char *hf = (c.hf_loss > 0.f && g.n > 1) ? P.hf_flag : nullptr;
     if (g.n > 1) {
         const int slots = hf ? strip_slots(SK_ROB_HF, (const void *)k_rob<true>)
@@ -280,10 +294,10 @@ cudaError_t launch_merge_prep_motion(const float *motion, const Geom &g, const M
 }
 
 cudaError_t launch_merge_prep(const uint16_t *burst, const float *motion, const Geom &g, const MergeConsts &c,
-                              const MergePlanes &P, cudaStream_t s) {
+                              const MergePlanes &P, cudaStream_t s, int snum, int sden) {
     const cudaError_t e = launch_merge_prep_frames(burst, g, c, P, s);
     if (e != cudaSuccess) return e;
-    return launch_merge_prep_motion(motion, g, c, P, s);
+    return launch_merge_prep_motion(motion, g, c, P, s, snum, sden);
 }
 
 cudaError_t launch_geo(const float *motion, const Geom &g, const MergePlanes &P, int snum, int sden, cudaStream_t s) {
@@ -294,12 +308,14 @@ cudaError_t launch_geo(const float *motion, const Geom &g, const MergePlanes &P,
 }
 
 cudaError_t launch_merge_accum(const uint16_t *burst, const float *motion, const Geom &g, const MergePlanes &P,
-                               int snum, int sden, float *rgb, float *den, cudaStream_t s) {
+                               int snum, int sden, float *rgb, float *den, bool have_geo, cudaStream_t s) {
     StageRange range("hmfsr merge: accumulation and normalisation");
     CheckedLaunches checked(s);
     const int ho = (int)(((long long)g.h * snum) / sden), wo = (int)(((long long)g.w * snum) / sden);
-    const cudaError_t e = launch_geo(motion, g, P, snum, sden, s);
-    if (e != cudaSuccess) return e;
+    if (!have_geo) {
+        const cudaError_t e = launch_geo(motion, g, P, snum, sden, s);
+        if (e != cudaSuccess) return e;
+    }
     if (den)
         launch_k_merge<true, false>(s, burst, g, P, snum, sden, ho, wo, rgb, den, stage::ChunkIO{});
     else
@@ -307,14 +323,12 @@ cudaError_t launch_merge_accum(const uint16_t *burst, const float *motion, const
     return cudaGetLastError();
 }
 
-cudaError_t launch_merge_accum_chunk(const uint16_t *burst, const float *motion, const Geom &g, const MergePlanes &P,
+cudaError_t launch_merge_accum_chunk(const uint16_t *burst, const Geom &g, const MergePlanes &P,
                                      int snum, int sden, float *rgb, float *den, const float *state_in,
                                      float *state_out, bool skip_base, cudaStream_t s) {
     StageRange range("hmfsr merge: accumulation of one chunk of frames");
     CheckedLaunches checked(s);
     const int ho = (int)(((long long)g.h * snum) / sden), wo = (int)(((long long)g.w * snum) / sden);
-    const cudaError_t e = launch_geo(motion, g, P, snum, sden, s);
-    if (e != cudaSuccess) return e;
     stage::ChunkIO io;
     io.state_in = state_in;
     io.state_out = state_out;

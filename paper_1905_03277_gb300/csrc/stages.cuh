@@ -1102,18 +1102,25 @@ __device__ __forceinline__ void prep_strip(const uint16_t *__restrict__ burst, c
 // motion prior (Eq. 7-8): robustness scale per tile, decided in exact FP64
 // --------------------------------------------------------------------------------------
 // the motion span M of tile (x, y) and its 3x3 tile neighbourhood exceeds m_th (Eq. 7);
-// min / max are exact in FP32; the span, its length and the threshold are FP64
+// min / max are exact in FP32 (a tile beyond the border is the border tile, which is in
+// the neighbourhood); the span, its length and the threshold are FP64 where FP32, six
+// roundings of 2^-24, does not already decide
 __device__ __forceinline__ bool motion_span_exceeds(const float2 *__restrict__ mv, int ty, int tx, int y, int x,
                                                     float m_th) {
     float mnx = INFINITY, mxx = -INFINITY, mny = INFINITY, mxy = -INFINITY;
+#pragma unroll
     for (int j = -1; j <= 1; ++j)
+#pragma unroll
         for (int k = -1; k <= 1; ++k) {
-            int yy = y + j, xx = x + k;
-            if (yy < 0 || yy >= ty || xx < 0 || xx >= tx) continue;
-            float2 v = HMFSR_LD(mv + (size_t)yy * tx + xx);
+            const float2 v = HMFSR_LD(mv + (size_t)clampi(y + j, 0, ty - 1) * tx + clampi(x + k, 0, tx - 1));
             mnx = fminf(mnx, v.x); mxx = fmaxf(mxx, v.x);
             mny = fminf(mny, v.y); mxy = fmaxf(mxy, v.y);
         }
+    if (m_th > 1e-6f && m_th < 1e6f) {
+        const float fx = mxx - mnx, fy = mxy - mny, len2 = fmaf(fx, fx, fy * fy), t2 = m_th * m_th;
+        if (len2 > t2 * 1.00001f) return true;
+        if (len2 < t2 * 0.99999f) return false;
+    }
     double Mx = __dsub_rn((double)mxx, (double)mnx), My = __dsub_rn((double)mxy, (double)mny);
     return length_exceeds(__dadd_rn(__dmul_rn(Mx, Mx), __dmul_rn(My, My)), m_th);
 }
