@@ -42,8 +42,10 @@ class MergeParams:
     tile: int = 16
 
     def c(self) -> _lib.MergeParamsC:
-        vals = [getattr(self, f.name) for f in fields(self) if f.name != "tile"]
-        return _lib.MergeParamsC(*[float(v) for v in vals], int(self.tile))
+        return _lib.MergeParamsC(float(self.k_detail), float(self.k_denoise), float(self.d_th), float(self.d_tr),
+                                 float(self.k_stretch), float(self.k_shrink), float(self.t), float(self.s1),
+                                 float(self.s2), float(self.m_th), float(self.noise_a), float(self.noise_b),
+                                 int(self.tile))
 
 
 @dataclass
@@ -97,30 +99,35 @@ def _merge_inputs(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams
 
 
 def _ptr(t: torch.Tensor | None):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None  # every pointer argument is declared as one
+
+
+def _on(device, stream):
+    """The stream a call runs on: the given one, or the device's current one."""
+    return stream if stream is not None else torch.cuda.current_stream(device)
 
 
 def _stream(device, stream):
-    s = stream if stream is not None else torch.cuda.current_stream(device)
-    return ctypes.c_void_p(s.cuda_stream)
+    return _on(device, stream).cuda_stream
 
 
 _ws_cache: dict = {}
 
 
-def _workspace(device: torch.device, nbytes: int, stream=None) -> torch.Tensor:
-    """A reusable, 256-byte aligned scratch buffer per (device, stream), grown on demand.
+def _workspace(device: torch.device, nbytes: int, stream) -> torch.Tensor:
+    """A reusable, 256-byte aligned scratch buffer per (device, stream), of at least nbytes,
+    grown on demand.
     Calls on one stream run in order and share it; calls on different streams get their
     own, so concurrent calls never race on scratch.  The buffer is allocated on that
     stream, so the caching allocator orders its reuse after the stream's work."""
-    s = stream if stream is not None else torch.cuda.current_stream(device)
-    key = (device.type, device.index, s.cuda_stream)
-    buf = _ws_cache.get(key)
-    if buf is None or buf.numel() < nbytes + 256:
-        with torch.cuda.stream(s):
-            _ws_cache[key] = buf = torch.empty(nbytes + 256, dtype=torch.uint8, device=device)
-    off = (-buf.data_ptr()) % 256
-    return buf[off:off + max(nbytes, 1)]
+    key = (device.type, device.index, stream.cuda_stream)
+    ws = _ws_cache.get(key)
+    if ws is None or ws.numel() < nbytes:
+        with torch.cuda.stream(stream):
+            buf = torch.empty(nbytes + 256, dtype=torch.uint8, device=device)
+        off = (-buf.data_ptr()) % 256
+        _ws_cache[key] = ws = buf[off:]
+    return ws
 
 
 def workspace_size(op: int, burst_shape, tile: int, scale=(1, 1), white_level: int = 4095) -> int:
@@ -139,6 +146,7 @@ def align(burst: torch.Tensor, ref: int = 0, params: AlignParams | None = None, 
     if not burst.is_cuda:
         raise ValueError("burst must be on a CUDA device")
     d = _desc(burst, ref, white_level)
+    stream = _on(burst.device, stream)
     n, h, w = burst.shape
     ty, tx = n_tiles(h, w, params.tile)
     motion = torch.empty((n, ty, tx, 2), dtype=torch.float32, device=burst.device)
@@ -150,7 +158,7 @@ def align(burst: torch.Tensor, ref: int = 0, params: AlignParams | None = None, 
         raise ValueError("subpixel must be 'lk' (Lucas-Kanade) or 'quadfit' (quadratic fit to the matching error)")
     fn = L.hmfsr_align if subpixel == "lk" else L.hmfsr_align_quadfit
     _lib.check(fn(_ptr(burst), ctypes.byref(d), ctypes.byref(pc), _ptr(motion), _ptr(mint), _ptr(ws), ws.numel(),
-                  _stream(burst.device, stream)), "hmfsr_align")
+                  stream.cuda_stream), "hmfsr_align")
     return (motion, mint) if with_int else motion
 
 
@@ -183,6 +191,7 @@ def merge(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams | None 
     L = _lib.load()
     params = params or MergeParams()
     d = _merge_inputs(burst, motion, params, ref, white_level)
+    stream = _on(burst.device, stream)
     n, h, w = burst.shape
     ho, wo = out_size(h, w, scale)
     rgb = torch.empty((3, ho, wo), dtype=torch.float32, device=burst.device)
@@ -192,7 +201,7 @@ def merge(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams | None 
         _workspace(burst.device, nbytes, stream)
     pc = params.c()
     _lib.check(L.hmfsr_merge(_ptr(burst), ctypes.byref(d), _ptr(motion), ctypes.byref(pc), scale[0], scale[1],
-                             _ptr(rgb), _ptr(den), _ptr(ws), ws.numel(), _stream(burst.device, stream)),
+                             _ptr(rgb), _ptr(den), _ptr(ws), ws.numel(), stream.cuda_stream),
                "hmfsr_merge")
     return (rgb, den) if with_den else rgb
 
@@ -205,6 +214,7 @@ def merge_chunked(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams
     L = _lib.load()
     params = params or MergeParams()
     d = _merge_inputs(burst, motion, params, ref, white_level)
+    stream = _on(burst.device, stream)
     n, h, w = burst.shape
     ho, wo = out_size(h, w, scale)
     rgb = torch.empty((3, ho, wo), dtype=torch.float32, device=burst.device)
@@ -216,7 +226,7 @@ def merge_chunked(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams
     pc = params.c()
     _lib.check(L.hmfsr_merge_chunked(_ptr(burst), ctypes.byref(d), _ptr(motion), ctypes.byref(pc), scale[0], scale[1],
                                      int(chunk_frames), _ptr(rgb), _ptr(den), _ptr(ws), ws.numel(),
-                                     _stream(burst.device, stream)), "hmfsr_merge_chunked")
+                                     stream.cuda_stream), "hmfsr_merge_chunked")
     return (rgb, den) if with_den else rgb
 
 
@@ -235,6 +245,7 @@ def merge_stages(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams 
     L = _lib.load()
     params = params or MergeParams()
     d = _merge_inputs(burst, motion, params, ref, white_level)
+    stream = _on(burst.device, stream)
     n, h, w = burst.shape
     omega = torch.empty((n, 3, h // 2, w // 2), dtype=torch.float32, device=burst.device)
     rhat = torch.empty((n, h // 2, w // 2), dtype=torch.float32, device=burst.device)
@@ -242,7 +253,7 @@ def merge_stages(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams 
     ws = _workspace(burst.device, nbytes, stream)
     pc = params.c()
     _lib.check(L.hmfsr_merge_stages(_ptr(burst), ctypes.byref(d), _ptr(motion), ctypes.byref(pc), _ptr(omega),
-                                    _ptr(rhat), _ptr(ws), ws.numel(), _stream(burst.device, stream)),
+                                    _ptr(rhat), _ptr(ws), ws.numel(), stream.cuda_stream),
                "hmfsr_merge_stages")
     return omega, rhat
 
@@ -267,6 +278,7 @@ def align_merge(burst: torch.Tensor, params: MergeParams | None = None, scale=(1
     ty, tx = n_tiles(h, w, params.tile)
     ho, wo = out_size(h, w, scale)
     dv = dev_burst.device
+    stream = _on(dv, stream)
     motion = torch.empty((n, ty, tx, 2), dtype=torch.float32, device=dv)
     if not host and out is not None:
         if not out.is_cuda or out.device != dv or out.dtype != torch.float32 or tuple(out.shape) != (3, ho, wo) \
@@ -282,7 +294,7 @@ def align_merge(burst: torch.Tensor, params: MergeParams | None = None, scale=(1
     ap, mp = align_params.c(), params.c()
     _lib.check(L.hmfsr_align_merge(_ptr(dev_burst), ctypes.byref(d), ctypes.byref(ap), ctypes.byref(mp), scale[0],
                                    scale[1], _ptr(motion), None, _ptr(rgb), None, _ptr(ws), ws.numel(),
-                                   _stream(dv, stream)), "hmfsr_align_merge")
+                                   stream.cuda_stream), "hmfsr_align_merge")
     if host:
         if out is None:
             out = torch.empty(rgb.shape, dtype=rgb.dtype, pin_memory=True)
@@ -419,6 +431,7 @@ def merge_noise(burst: torch.Tensor, motion: torch.Tensor, table: torch.Tensor, 
     L = _lib.load()
     params = params or MergeParams()
     d = _merge_inputs(burst, motion, params, ref, white_level, table)
+    stream = _on(burst.device, stream)
     if table.dtype != torch.float32 or tuple(table.shape) != (_lib.NOISE_LEVELS, 4) or not table.is_contiguous():
         raise ValueError(f"noise table must be contiguous float32 [{_lib.NOISE_LEVELS},4]")
     n, h, w = burst.shape
@@ -429,7 +442,7 @@ def merge_noise(burst: torch.Tensor, motion: torch.Tensor, table: torch.Tensor, 
     ws = _workspace(burst.device, nbytes, stream)
     pc = params.c()
     _lib.check(L.hmfsr_merge_noise(_ptr(burst), ctypes.byref(d), _ptr(motion), ctypes.byref(pc), _ptr(table), scale[0],
-                                   scale[1], _ptr(rgb), _ptr(den), _ptr(ws), ws.numel(), _stream(burst.device, stream)),
+                                   scale[1], _ptr(rgb), _ptr(den), _ptr(ws), ws.numel(), stream.cuda_stream),
                "hmfsr_merge_noise")
     return (rgb, den) if with_den else rgb
 
@@ -443,6 +456,7 @@ def merge_ex(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams | No
     L = _lib.load()
     params = params or MergeParams()
     d = _merge_inputs(burst, motion, params, ref, white_level, noise_table)
+    stream = _on(burst.device, stream)
     if noise_table is not None and (noise_table.dtype != torch.float32 or not noise_table.is_contiguous()
                                     or tuple(noise_table.shape) != (_lib.NOISE_LEVELS, 4)):
         raise ValueError(f"noise table must be contiguous float32 [{_lib.NOISE_LEVELS},4]")
@@ -456,7 +470,7 @@ def merge_ex(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams | No
     opts = _lib.MergeOptionsC(noise_table.data_ptr() if noise_table is not None else None, float(hf_loss))
     _lib.check(L.hmfsr_merge_ex(_ptr(burst), ctypes.byref(d), _ptr(motion), ctypes.byref(pc), ctypes.byref(opts),
                                 scale[0], scale[1], _ptr(rgb), _ptr(den), _ptr(ws), ws.numel(),
-                                _stream(burst.device, stream)), "hmfsr_merge_ex")
+                                stream.cuda_stream), "hmfsr_merge_ex")
     return (rgb, den) if with_den else rgb
 
 
@@ -470,6 +484,7 @@ def merge_prepare(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams
     L = _lib.load()
     params = params or MergeParams()
     d = _merge_inputs(burst, motion, params, ref, white_level, workspace)
+    stream = _on(burst.device, stream)
     nbytes = L.hmfsr_workspace_size(_lib.OP_MERGE_STAGES, ctypes.byref(d), params.tile, 1, 1)
     if workspace is None:
         s = stream if stream is not None else torch.cuda.current_stream(burst.device)
@@ -485,7 +500,7 @@ def merge_prepare(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams
         ws = workspace
     pc = params.c()
     _lib.check(L.hmfsr_merge_prepare(_ptr(burst), ctypes.byref(d), _ptr(motion), ctypes.byref(pc), _ptr(ws),
-                                     ws.numel(), _stream(burst.device, stream)), "hmfsr_merge_prepare")
+                                     ws.numel(), stream.cuda_stream), "hmfsr_merge_prepare")
     return ws
 
 
@@ -496,6 +511,7 @@ def merge_accumulate(burst: torch.Tensor, motion: torch.Tensor, ws: torch.Tensor
     L = _lib.load()
     params = params or MergeParams()
     d = _merge_inputs(burst, motion, params, ref, white_level, ws, out, den)
+    stream = _on(burst.device, stream)
     n, h, w = burst.shape
     ho, wo = out_size(h, w, scale)
     nbytes = L.hmfsr_workspace_size(_lib.OP_MERGE_STAGES, ctypes.byref(d), params.tile, 1, 1)
@@ -509,7 +525,7 @@ def merge_accumulate(burst: torch.Tensor, motion: torch.Tensor, ws: torch.Tensor
     pc = params.c()
     _lib.check(L.hmfsr_merge_accumulate(_ptr(burst), ctypes.byref(d), _ptr(motion), ctypes.byref(pc), scale[0],
                                         scale[1], _ptr(out), _ptr(den), _ptr(ws), ws.numel(),
-                                        _stream(burst.device, stream)), "hmfsr_merge_accumulate")
+                                        stream.cuda_stream), "hmfsr_merge_accumulate")
     return out
 
 
@@ -544,12 +560,13 @@ def merge_static(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams 
     L = _lib.load()
     params = params or MergeParams()
     d = _merge_inputs(burst, motion, params, ref, white_level)
+    stream = _on(burst.device, stream)
     n, h, w = burst.shape
     ho, wo = out_size(h, w, scale)
     rgb = torch.empty((3, ho, wo), dtype=torch.float32, device=burst.device)
     pc = params.c()
     _lib.check(L.hmfsr_merge_static(_ptr(burst), ctypes.byref(d), _ptr(motion), ctypes.byref(pc), scale[0], scale[1],
-                                    _ptr(rgb), None, _stream(burst.device, stream)), "hmfsr_merge_static")
+                                    _ptr(rgb), None, stream.cuda_stream), "hmfsr_merge_static")
     return rgb
 
 
@@ -568,6 +585,7 @@ def merge_backward(burst: torch.Tensor, motion: torch.Tensor, params: MergeParam
         raise ValueError("prepared=True needs the forward's workspace")
     L = _lib.load()
     d = _merge_inputs(burst, motion, params, ref, white_level, rgb, den, grad_rgb)
+    stream = _on(burst.device, stream)
     n, h, w = burst.shape
     ty, tx = n_tiles(h, w, params.tile)
     ho, wo = out_size(h, w, scale)
@@ -586,7 +604,7 @@ def merge_backward(burst: torch.Tensor, motion: torch.Tensor, params: MergeParam
     pc = params.c()
     fn = L.hmfsr_merge_backward_prepared if prepared else L.hmfsr_merge_backward
     _lib.check(fn(_ptr(burst), ctypes.byref(d), _ptr(motion), ctypes.byref(pc), scale[0], scale[1], _ptr(rgb),
-                  _ptr(den), _ptr(grad_rgb), _ptr(gp), _ptr(gm), _ptr(ws), ws.numel(), _stream(burst.device, stream)),
+                  _ptr(den), _ptr(grad_rgb), _ptr(gp), _ptr(gm), _ptr(ws), ws.numel(), stream.cuda_stream),
                "hmfsr_merge_backward")
     return gp, gm
 
