@@ -507,7 +507,7 @@ def run_gpu(args):
         fma, ex2 = pipe_peaks["fp32_fma"], pipe_peaks["mufu_ex2"]
         peak = fma["lane_ops_per_s"] / 1e12
         mufu_peak = ex2["lane_ops_per_s"] / 1e12
-        roof = {"bound": "alu", "kernel": "k_merge_q1 (hmfsr_merge_accumulate: k_geo, k_merge_q1)", "achieved": achieved, "peak": peak,
+        roof = {"bound": "alu", "kernel": "k_merge_region (hmfsr_merge_accumulate: k_geo, k_merge_region)", "achieved": achieved, "peak": peak,
                 "unit": "T lane-ops/s", "frac": achieved / peak, "traffic": kernel_traffic("k_merge_12mp"),
                 "peak_source": (f"measured: FP32 FMA issue rate of hmfsr_pipe_probe on this GPU ({n_sm} SMs, "
                                 f"{fma['sm_mhz']} MHz sampled; {fma['per_sm_per_clk']:.1f} lane-ops per SM per clock)"),
@@ -529,6 +529,7 @@ def run_gpu(args):
                    "sample": f"the whole step once: oracle alignment of the 8-frame 12-MP burst ({t_align:.2f} s) "
                              f"+ oracle merge of all {ho} output rows ({t_merge:.2f} s)"}
         per_call = hm.launches_per_call(n, h, w, ap.n_levels, ap.tile, ap.radius[0])
+        per_call["merge_accumulate"] -= 1  # in the one call the window geometry goes with the motion strength
         launches = args.steps * sum(per_call.values())
         merge_only_ms = statistics.median([p_ + a_ for p_, a_ in zip(prep_ms, acc_ms)])
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,

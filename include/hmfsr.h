@@ -290,7 +290,8 @@ hmfsr_status hmfsr_batch_vectors(hmfsr_batch_plan plan, const void *ws, int burs
                                  void *stream);
 
 /* Settings: accumulation work item of merge_tile_w x (128 / merge_tile_w) output pixels
- * (merge_tile_w divides 128), ctas_per_sm persistent blocks per SM (0 = as many as fit),
+ * (merge_tile_w divides 128; scales 1, 3/2 and 2 with tiles of 16 px and more take 16 x 16
+ * raw px regions whatever it is), ctas_per_sm persistent blocks per SM (0 = as many as fit),
  * regs_variant (kernel build with 0: 128, 1: 80, 2: 64 registers per thread),
  * queue_order (0: stage-major, 1: burst-major, 2: wavefront), spin_limit polls per dependency wait
  * before HMFSR_ERR_TIMEOUT, and inject_stall != 0 to add a dependency nothing satisfies
@@ -303,8 +304,8 @@ hmfsr_status hmfsr_batch_configure(hmfsr_batch_plan plan, int merge_tile_w, int 
 hmfsr_status hmfsr_batch_set_mode(hmfsr_batch_plan plan, int streams);
 
 /* Autotuner: times the batch on the given buffers for 8 candidates -- the persistent
- * kernel at 128 registers per thread with accumulation tiles 32x4 and 16x8 (for scales
- * other than 1; scale 1 always takes 2 x 2 pixel blocks), at 80 and at 64 registers
+ * kernel at 128 registers per thread with accumulation tiles 32x4 and 16x8 (where they
+ * apply: hmfsr_batch_configure), at 80 and at 64 registers
  * (32x4), and at 128 registers with the wavefront queue; and the per-burst graph on 2, 4
  * and 8 branches -- keeps the fastest in the plan and returns its time (ms) in *best_ms
  * and every candidate's time in tune_log[8] (both nullable).  Overwrites the outputs. */

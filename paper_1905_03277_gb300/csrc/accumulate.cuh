@@ -394,6 +394,7 @@ __device__ __forceinline__ void merge_px(const uint16_t *__restrict__ burst, con
 // ======================================================================================
 // accumulation at scale 1 (Eq. 1-2): one thread per 2 x NY block of output pixels
 // ======================================================================================
+// (8-px motion tiles; larger ones take accumulate_region.cuh.)
 // At scale 1 output pixel X sits at raw x0 = X and the motion tile is chosen by the base
 // position, so the pixels of an even-aligned 2 x NY block lie in one tile and share the
 // frame's motion v.  Their window centres are (kx, ky) + (pa, pb) with kx = X + round(vx),

@@ -15,8 +15,8 @@
 // What bounds it: issue and shared-memory bandwidth, 12 MP x 8 at scale 1: ~225 warp-instructions
 // per 32 pixel-frames (the 2 x 2-pixel kernel it replaces: 271), issue 60 %, shared-memory data
 // path 80 %; DRAM 10 %.  One box, accumulation call:
-//   12 MP x 8, 1x    1147 -> 930 us      12 MP x 8, 1.5x   2756 -> 1920 us
-//   12 MP x 15, 2x   8568 -> 5315 us     0.07 MP x 8, 1x     57 -> 40 us
+//   12 MP x 8, 1x    1147 -> 916 us      12 MP x 8, 1.5x   2756 -> 1947 us
+//   12 MP x 15, 2x   8568 -> 5320 us     0.07 MP x 8, 1x     57 -> 38 us
 #pragma once
 
 #include <limits.h>

@@ -6,7 +6,8 @@
 // tiles, s1/s2 selection, clamps, the 5x5 argmin, bilinear cells) carry no gradient.
 // The forward is recomputed from the burst; the forward's normalised colour C and
 // log2 of its weight sum are read back, so each sample's normalised weight is
-// 2^-(q' + log2 den).  All reductions are deterministic: per-pixel and per-texel
+// 2^-(q' + log2 den).  At scales 1, 3/2 and 2 with tiles of 16 px and more the per-pixel kernels
+// here give way to merge_bwd_region.cu.  All reductions are deterministic: per-pixel and per-texel
 // contributions go to buffers and are summed in a fixed order in FP64.
 #include "adjoint_common.cuh"
 

@@ -112,7 +112,7 @@ struct NoiseLevel {
 // Their truncation (12 x 16 x 2^-32 = 4.5e-8), the conversion and the two roundings are below
 // 4e-7 |w| + 2e-7 sigma + 1e-6 of w; only a w closer than that to a whole number (1 sample in
 // 10^4) takes the FP64 sequence, which this GPU issues at 1/64 of the FP32 rate.  All 28.5 M
-// samples in FP64: 863 us; now 1/7 of that or less, bound by the Philox integer products.
+// samples in FP64: 863 us; now 259, bound by the Philox integer products.
 __device__ __forceinline__ int noise_sample(const NoiseLevel &n, int trial, int j) {
     uint32_t s = 0;
 #pragma unroll
