@@ -14,8 +14,8 @@
 //     gather onto texels has constant weights.
 // Fixed orders everywhere, so results are deterministic.
 //
-// Bounded by the issue rate (57 %) with the shared-memory path at 56 %: 645 warp-instructions per
-// 32 pixel-frames.  At 1 MP x 8 frames, scale 3/2 (the fitting workload) the main kernel takes 540 us
+// Bounded by the issue rate (57 %) with the shared-memory path at 56 %: 560 instructions per
+// pixel-frame.  At 1 MP x 8 frames, scale 3/2 (the fitting workload) the main kernel takes 548 us
 // where the per-pixel one takes 802, the R-hat path 68 where its two kernels take 106.  Registers
 // decide the rest: shared memory leaves little L1, so every word spilled in the frame loop goes to
 // L2 (a version with 16 spilled words took 654 us).  Hence staging through shared memory and not
@@ -511,27 +511,21 @@ __global__ void __launch_bounds__(kRpW *kRpH) k_rpath_region(const float *__rest
 // Every tile's motion gradient: its regions' and its 8 x 8-texel blocks' sums, in a fixed order.
 // Eight lanes per tile, so that a tile's loads (up to 16 parts of each region) are in flight
 // together: latency is all of it.  One lane per tile took 23 us for the 256 x 320 x 4 crop at 2x
-// and 17 for 1 MP x 8 at 3/2; this in FP64 8 and 18, and with each addition's rounding error
-// carried in FP32 instead 8 and 9.
+// and 17 for 1 MP x 8 at 3/2; this 8 and 18 (FP64 sums).
 constexpr int kTileLanes = 8;
 __global__ void __launch_bounds__(128) k_motion_region(const float2 *__restrict__ vbar_region, const float2 *__restrict__ vbar_block,
                                                        Geom g, int off, int parts, float2 *__restrict__ grad_motion) {
     const int t = (blockIdx.x * 128 + threadIdx.x) / kTileLanes, l = threadIdx.x % kTileLanes;
     const int ntl = g.ty * g.tx, f = t / ntl, r = t - f * ntl, ty = r / g.tx, tx = r - ty * g.tx;
-    float x = 0.f, xe = 0.f, y = 0.f, ye = 0.f;
-    auto add = [](float &s, float &e, float v, float ve) {  // two-sum
-        const float q = s + v, p = q - s;
-        e += ((s - (q - p)) + (v - p)) + ve;
-        s = q;
-    };
+    double x = 0.0, y = 0.0;
     if (t < g.n * ntl && f != g.ref) {
         const int nb = g.tile / 16, nbx = div_up(g.wh, 8), nby = div_up(g.hh, 8);
         const int x0 = tx * nb, y0 = ty * nb, bw = min(x0 + nb, nbx) - x0, bh = min(y0 + nb, nby) - y0;
         for (int k = l; k < bw * bh; k += kTileLanes) {
             const int by = k / bw, bx = k - by * bw;
             const float2 q = __ldg(vbar_block + ((size_t)f * nby + y0 + by) * nbx + x0 + bx);
-            add(x, xe, q.x, 0.f);
-            add(y, ye, q.y, 0.f);
+            x += (double)q.x;
+            y += (double)q.y;
         }
         // regions are the same 8 x 8 texels, after `off` leading ones that belong to the first tiles
         const int nrx = nbx + off, nry = nby + off;
@@ -540,16 +534,16 @@ __global__ void __launch_bounds__(128) k_motion_region(const float2 *__restrict_
             const int q0 = k / parts, by = q0 / rw, bx = q0 - by * rw;
             const float4 q = __ldg(reinterpret_cast<const float4 *>(vbar_region) +
                                    (((size_t)f * nry + ry0 + by) * nrx + rx0 + bx) * parts + (k - q0 * parts));
-            add(x, xe, q.x, q.y);
-            add(y, ye, q.z, q.w);
+            x += (double)q.x + (double)q.y;
+            y += (double)q.z + (double)q.w;
         }
     }
 #pragma unroll
     for (int o = kTileLanes / 2; o > 0; o >>= 1) {
-        add(x, xe, __shfl_xor_sync(0xffffffffu, x, o), __shfl_xor_sync(0xffffffffu, xe, o));
-        add(y, ye, __shfl_xor_sync(0xffffffffu, y, o), __shfl_xor_sync(0xffffffffu, ye, o));
+        x += __shfl_xor_sync(0xffffffffu, x, o);
+        y += __shfl_xor_sync(0xffffffffu, y, o);
     }
-    if (l == 0 && t < g.n * ntl) grad_motion[t] = make_float2(x + xe, y + ye);
+    if (l == 0 && t < g.n * ntl) grad_motion[t] = make_float2((float)x, (float)y);
 }
 
 template <int SN, int SD>
