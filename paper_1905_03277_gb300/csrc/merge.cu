@@ -12,8 +12,9 @@ namespace {
 using stage::kMergeW;
 using stage::kMergeH;
 
-// 4 warps side by side: 128 texel columns x `rows` rows of frame f0 + blockIdx.z
-__global__ void __launch_bounds__(128) k_prep(const uint16_t *__restrict__ burst, Geom g, MergeConsts c,
+// 4 warps side by side: 128 texel columns x `rows` rows of frame f0 + blockIdx.z.  8 blocks per SM
+// (64 registers): 7 take 2 us more at 12 MP x 8 frames, 10 (spills) 14, 6 10.
+__global__ void __launch_bounds__(128, 8) k_prep(const uint16_t *__restrict__ burst, Geom g, MergeConsts c,
                                               uint2 *__restrict__ s1, float4 *__restrict__ base_stats,
                                               float4 *__restrict__ kern, int rows, int f0) {
     stage::prep_strip(burst, g, c, s1, base_stats, kern, blockIdx.x * 128 + (threadIdx.x & ~31),

@@ -922,20 +922,22 @@ __device__ __forceinline__ float4 base_stats_of(const uint32_t (&S1)[3], const u
 
 // --------------------------------------------------------------------------------------
 // structure tensor -> kernel covariance (Eq. 3, Eq. 4, supplement S.1), from the exact
-// integer tensor {sum gx^2, sum gx gy, sum gy^2} of the four 2x2 sub-squares
+// integer tensor of the four 2x2 sub-squares (a b over c d) by their diagonal differences
+// p = d - a and q = b - c: gx = p + q and gy = p - q, so with pp, qq and pq the sums of p^2, q^2
+// and p q the trace is 2 (pp + qq), gx^2 - gy^2 is 4 pq and gx gy is pp - qq
 // --------------------------------------------------------------------------------------
 // inv_dtr = 1 / (16 WL D_tr)
-__device__ __forceinline__ float4 kern_of_tensor(long long ta, long long tb, long long tc, const MergeConsts &c,
+__device__ __forceinline__ float4 kern_of_tensor(long long pp, long long qq, long long pq, const MergeConsts &c,
                                                  float inv_dtr) {
     // eigen-analysis: lambda1 = (tr + r)/2, dominant direction at angle theta with
     // cos 2theta = (a-c)/r, sin 2theta = 2b/r (theta = 0 when the tensor is isotropic)
-    float tr = (float)(ta + tc);
-    float amc = (float)(ta - tc), b2 = 2.f * (float)tb;
+    float tr = 2.f * (float)(pp + qq);
+    float amc = 4.f * (float)pq, b2 = 2.f * (float)(pp - qq);  // exact values, each rounded once
     float r = fast_sqrt(fmaf(amc, amc, b2 * b2));
     float cs = 1.f, sn = 0.f;
-    if (!(ta == tc && tb == 0)) { const float ir = fast_rcp(r); cs = amc * ir; sn = b2 * ir; }
+    if (!(pq == 0 && pp == qq)) { const float ir = fast_rcp(r); cs = amc * ir; sn = b2 * ir; }
     float l1 = 0.5f * (tr + r);
-    float A = (ta + tc == 0) ? 1.f : 1.f + fast_sqrt(r * fast_rcp(tr));
+    float A = (tr == 0.f) ? 1.f : 1.f + fast_sqrt(r * fast_rcp(tr));
     // lambda in units of luminance normalised to [0,1]: sqrt(l1_norm) = sqrt(l1) / (16 WL)
     float D = fminf(fmaxf(fmaf(-fast_sqrt(l1), inv_dtr, 1.f) + c.d_th, 0.f), 1.f);
     float kh_al = c.k_detail * (c.k_stretch * A);
@@ -985,7 +987,7 @@ struct PrepState {
     uint32_t rb[2], gs[2];  // 3-texel row sums of the two previous rows: R | B << 16, G1 + G2
     uint32_t q[2][3];       // 3-texel row sums of squares (base frame)
     int L[3];               // Lq of the previous row at columns -1, 0, +1
-    long long pa, pb, pc;   // tensor terms of the previous pair of rows
+    long long pp, qq, pq;   // tensor terms of the previous pair of rows
 };
 
 __device__ __forceinline__ PrepRow prep_fetch(const uint16_t *__restrict__ fr, int pitch, int hh, int uc, int uh,
@@ -1002,8 +1004,11 @@ __device__ __forceinline__ PrepRow prep_fetch(const uint16_t *__restrict__ fr, i
     return p;
 }
 
-// one raw row pair of the strip (strip row r = -1 .. rows); emits texel row r - 1
-__device__ __forceinline__ void prep_row(const PrepRow &p, PrepState &st, int r, int lane, bool is_ref, bool out_col,
+// one raw row pair of the strip (strip row r = -1 .. rows); emits texel row r - 1.  kRef: the
+// base frame, whose squares the others neither sum nor carry along (as a run-time test it cost
+// the others branches and 6 registers: 12 MP x 8 frames 182 us, so 172)
+template <bool kRef>
+__device__ __forceinline__ void prep_row(const PrepRow &p, PrepState &st, int r, int lane, bool out_col,
                                          int v0, const Geom &g, const MergeConsts &c, float inv_dtr, int u,
                                          uint2 *__restrict__ s1f, float4 *__restrict__ base_stats,
                                          float4 *__restrict__ kernf) {
@@ -1024,7 +1029,7 @@ __device__ __forceinline__ void prep_row(const PrepRow &p, PrepState &st, int r,
     const uint32_t gs = (l1 & 0xffffu) + G + (r1 & 0xffffu);
     const int L[3] = {(int)(l1 >> 16), (int)(c1 >> 16), (int)(r1 >> 16)};
     uint32_t q[3] = {0u, 0u, 0u};
-    if (is_ref) {
+    if (kRef) {
         const uint32_t lR = l0 & 0xffffu, lB = l0 >> 16, lG = l1 & 0xffffu;
         const uint32_t rR = r0 & 0xffffu, rB = r0 >> 16, rG = r1 & 0xffffu;
         q[0] = lR * lR + R * R + rR * rR;
@@ -1032,14 +1037,13 @@ __device__ __forceinline__ void prep_row(const PrepRow &p, PrepState &st, int r,
         q[2] = lB * lB + B * B + rB * rB;
     }
     // tensor terms of the two sub-squares between the previous row and this one
-    long long pa = 0, pb = 0, pc = 0;
+    long long pp = 0, qq = 0, pq = 0;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-        const int gx = (st.L[i + 1] - st.L[i]) + (L[i + 1] - L[i]);
-        const int gy = (L[i] - st.L[i]) + (L[i + 1] - st.L[i + 1]);
-        pa += (long long)gx * gx;
-        pb += (long long)gx * gy;
-        pc += (long long)gy * gy;
+        const int dp = L[i + 1] - st.L[i], dq = st.L[i + 1] - L[i];
+        pp += (long long)dp * dp;
+        qq += (long long)dq * dq;
+        pq += (long long)dp * dq;
     }
     if (r >= 1 && out_col) {
         const int v = v0 + r - 1;
@@ -1047,22 +1051,23 @@ __device__ __forceinline__ void prep_row(const PrepRow &p, PrepState &st, int r,
             const int idx = v * g.wh + u;
             const uint32_t srb = st.rb[0] + st.rb[1] + rb, sg = st.gs[0] + st.gs[1] + gs;
             HMFSR_ST(s1f + idx, make_uint2(srb, sg));
-            if (is_ref) {
+            if (kRef) {
                 const uint32_t S1[3] = {srb & 0xffffu, sg, srb >> 16};
                 const uint32_t S2[3] = {st.q[0][0] + st.q[1][0] + q[0], st.q[0][1] + st.q[1][1] + q[1],
                                         st.q[0][2] + st.q[1][2] + q[2]};
                 HMFSR_ST(base_stats + idx, base_stats_of(S1, S2, c, g.wl));
             }
-            HMFSR_ST(kernf + idx, kern_of_tensor(st.pa + pa, st.pb + pb, st.pc + pc, c, inv_dtr));
+            HMFSR_ST(kernf + idx, kern_of_tensor(st.pp + pp, st.qq + qq, st.pq + pq, c, inv_dtr));
         }
     }
     st.rb[0] = st.rb[1]; st.rb[1] = rb;
     st.gs[0] = st.gs[1]; st.gs[1] = gs;
+    if (kRef)
 #pragma unroll
-    for (int ch = 0; ch < 3; ++ch) { st.q[0][ch] = st.q[1][ch]; st.q[1][ch] = q[ch]; }
+        for (int ch = 0; ch < 3; ++ch) { st.q[0][ch] = st.q[1][ch]; st.q[1][ch] = q[ch]; }
 #pragma unroll
     for (int i = 0; i < 3; ++i) st.L[i] = L[i];
-    st.pa = pa; st.pb = pb; st.pc = pc;
+    st.pp = pp; st.qq = qq; st.pq = pq;
 }
 
 // strip (u0 .. u0 + 31) x (v0 .. v0 + rows - 1) of frame f (rows even); every lane of the
@@ -1075,7 +1080,7 @@ __device__ __forceinline__ void prep_strip(const uint16_t *__restrict__ burst, c
     const int u = u0 + lane, uc = min(u, g.wh - 1);
     const bool halo = (lane == 0 || lane == 31);
     const int uh = clampi(lane == 0 ? u0 - 1 : u0 + 32, 0, g.wh - 1);
-    const bool is_ref = (f == g.ref), out_col = u < g.wh;
+    const bool out_col = u < g.wh;
     const size_t hw = (size_t)g.hh * g.wh;
     uint2 *s1f = s1 + (size_t)f * hw;
     float4 *kernf = kern + (size_t)f * hw;
@@ -1085,17 +1090,23 @@ __device__ __forceinline__ void prep_strip(const uint16_t *__restrict__ burst, c
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch) st.q[0][ch] = st.q[1][ch] = 0u;
     st.L[0] = st.L[1] = st.L[2] = 0;
-    st.pa = st.pb = st.pc = 0;
+    st.pp = st.qq = st.pq = 0;
     PrepRow p0 = prep_fetch(fr, g.pitch, g.hh, uc, uh, halo, v0 - 1);
     PrepRow p1 = prep_fetch(fr, g.pitch, g.hh, uc, uh, halo, v0);
-    for (int r = -1; r <= rows; r += 2) {
-        const PrepRow cur0 = p0;
-        p0 = prep_fetch(fr, g.pitch, g.hh, uc, uh, halo, v0 + r + 2);
-        prep_row(cur0, st, r, lane, is_ref, out_col, v0, g, c, inv_dtr, u, s1f, base_stats, kernf);
-        const PrepRow cur1 = p1;
-        p1 = prep_fetch(fr, g.pitch, g.hh, uc, uh, halo, v0 + r + 3);
-        prep_row(cur1, st, r + 1, lane, is_ref, out_col, v0, g, c, inv_dtr, u, s1f, base_stats, kernf);
-    }
+    auto walk = [&](auto row) {
+        for (int r = -1; r <= rows; r += 2) {
+            const PrepRow cur0 = p0;
+            p0 = prep_fetch(fr, g.pitch, g.hh, uc, uh, halo, v0 + r + 2);
+            row(cur0, r);
+            const PrepRow cur1 = p1;
+            p1 = prep_fetch(fr, g.pitch, g.hh, uc, uh, halo, v0 + r + 3);
+            row(cur1, r + 1);
+        }
+    };
+    if (f == g.ref)
+        walk([&](const PrepRow &p, int r) { prep_row<true>(p, st, r, lane, out_col, v0, g, c, inv_dtr, u, s1f, base_stats, kernf); });
+    else
+        walk([&](const PrepRow &p, int r) { prep_row<false>(p, st, r, lane, out_col, v0, g, c, inv_dtr, u, s1f, base_stats, kernf); });
 }
 
 // --------------------------------------------------------------------------------------
