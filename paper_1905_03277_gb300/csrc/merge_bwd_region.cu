@@ -14,8 +14,8 @@
 //     gather onto texels has constant weights.
 // Fixed orders everywhere, so results are deterministic.
 //
-// Bounded by the issue rate (57 %) with the shared-memory path at 56 %: 560 instructions per
-// pixel-frame.  At 1 MP x 8 frames, scale 3/2 (the fitting workload) the main kernel takes 548 us
+// Bounded by the issue rate (57 %) with the shared-memory path at 56 %: 645 warp-instructions per
+// 32 pixel-frames.  At 1 MP x 8 frames, scale 3/2 (the fitting workload) the main kernel takes 540 us
 // where the per-pixel one takes 802, the R-hat path 68 where its two kernels take 106.  Registers
 // decide the rest: shared memory leaves little L1, so every word spilled in the frame loop goes to
 // L2 (a version with 16 spilled words took 654 us).  Hence staging through shared memory and not
@@ -511,7 +511,8 @@ __global__ void __launch_bounds__(kRpW *kRpH) k_rpath_region(const float *__rest
 // Every tile's motion gradient: its regions' and its 8 x 8-texel blocks' sums, in a fixed order.
 // Eight lanes per tile, so that a tile's loads (up to 16 parts of each region) are in flight
 // together: latency is all of it.  One lane per tile took 23 us for the 256 x 320 x 4 crop at 2x
-// and 17 for 1 MP x 8 at 3/2; this 8 and 18 (FP64 sums).
+// and 17 for 1 MP x 8 at 3/2; this 8 and 18 (FP64 sums:
+// FP32 with the rounding errors carried took 9, but makes an infinite sum a NaN).
 constexpr int kTileLanes = 8;
 __global__ void __launch_bounds__(128) k_motion_region(const float2 *__restrict__ vbar_region, const float2 *__restrict__ vbar_block,
                                                        Geom g, int off, int parts, float2 *__restrict__ grad_motion) {
