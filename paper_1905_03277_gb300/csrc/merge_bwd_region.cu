@@ -405,7 +405,8 @@ __global__ void __launch_bounds__(kRpW *kRpH) k_rpath_region(const float *__rest
     const size_t plane = (size_t)(g.hh + kOff) * wg;
     const float *Pf = rhbar_phase + (size_t)f * (S * S) * plane;
     // along x, for each y phase: the pixel rows that the taps of texel rows v0 - 2 .. v0 + kRpH + 1
-    // touch.  Away from the border a phase's two taps and weights are constants.
+    // touch.  Away from the border a phase's two taps and weights are constants.  A pixel of weight 0
+    // is left out, so that one without a finite gradient reaches no texel that it does not sample.
     constexpr int kRows = kRpHaloH + 1;
     constexpr float inv2Q = 0.25f / (float)SN;
     for (int i = threadIdx.x; i < S * kRows * kRpHaloW; i += kRpW * kRpH) {
@@ -422,7 +423,8 @@ __global__ void __launch_bounds__(kRpW *kRpH) k_rpath_region(const float *__rest
                     int rc;
                     const float w = (float)stage::region_phase<SN, SD>(sx, rc) * inv2Q;
                     const float *ps = p + (size_t)sx * plane + (uu - rc + kOff);
-                    acc = fmaf(1.f - w, __ldg(ps), fmaf(w, __ldg(ps - 1), acc));
+                    if (w != 0.f) acc = fmaf(w, __ldg(ps - 1), acc);
+                    acc = fmaf(1.f - w, __ldg(ps), acc);
                 }
             } else {
 #pragma unroll
@@ -431,7 +433,8 @@ __global__ void __launch_bounds__(kRpW *kRpH) k_rpath_region(const float *__rest
                     float wx[2];
                     rhat_phase_taps<SN, SD>(uu, g.wh, sx, ix, wx);
                     const float *ps = p + (size_t)sx * plane;
-                    acc = fmaf(wx[0], __ldg(ps + ix[0]), fmaf(wx[1], __ldg(ps + ix[1]), acc));
+                    if (wx[1] != 0.f) acc = fmaf(wx[1], __ldg(ps + ix[1]), acc);
+                    if (wx[0] != 0.f) acc = fmaf(wx[0], __ldg(ps + ix[0]), acc);
                 }
             }
         }
@@ -450,7 +453,8 @@ __global__ void __launch_bounds__(kRpW *kRpH) k_rpath_region(const float *__rest
                 int iy[2];
                 float wy[2];
                 rhat_phase_taps<SN, SD>(vv, g.hh, sy, iy, wy);
-                acc = fmaf(wy[0], s_x[sy][r + 1][cc], fmaf(wy[1], s_x[sy][r][cc], acc));
+                if (wy[1] != 0.f) acc = fmaf(wy[1], s_x[sy][r][cc], acc);
+                if (wy[0] != 0.f) acc = fmaf(wy[0], s_x[sy][r + 1][cc], acc);
             }
         }
         s_rh[r][cc] = make_float2(acc, __int_as_float(fl));
