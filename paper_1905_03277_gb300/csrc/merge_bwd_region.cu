@@ -243,8 +243,9 @@ __global__ void __launch_bounds__(32 * AdjointShape<SN, SD>::kSy *RegionScale<SN
                         if (!(xok[i] && yok[j])) w.x = 0.f;
                         if (!(xok[i] && yok[j + 2])) w.y = 0.f;
                     }
-                    const float2 e = mul2(fma2(G[k], make_float2(val[j], val[j + 2]), nGC[k]), w);  // dL/d(w Rhat) w
-                    rhb = add2(rhb, e);
+                    const float2 gv = fma2(G[k], make_float2(val[j], val[j + 2]), nGC[k]);  // dL/d(w Rhat)
+                    rhb = fma2(gv, w, rhb);
+                    const float2 e = mul2(gv, mul2(w, rh));  // times w Rhat, which is at most 1
                     const float2 t1 = mul2(e, Px), t2 = mul2(e, Py);
                     sPx = add2(sPx, t1);
                     sPy = add2(sPy, t2);
@@ -253,18 +254,21 @@ __global__ void __launch_bounds__(32 * AdjointShape<SN, SD>::kSy *RegionScale<SN
                     o11 = fma2(t2, Py, o11);
                 }
             }
-            // Omega-bar = Rhat / 2 sum e P P^T (o01 doubled: the entry stands for both); the offsets
-            // give dL/dv = Rhat sum e P
-            const float2 hr = mul2(make_float2(0.5f, 0.5f), rh);
-            o00 = mul2(o00, hr);
-            o11 = mul2(o11, hr);
-            o01 = mul2(o01, rh);
+            // Omega-bar = sum e P P^T / 2 (o01 doubled: the entry stands for both); the offsets give
+            // dL/dv = sum e P.  A frame rejected at a pixel is not in its channels' sums, so its w has
+            // no bound: it is left out here, where 0 times it (or times its product with P) may be no
+            // number.
+            const float2 half = make_float2(0.5f, 0.5f);
+            o00 = mul2(o00, half);
+            o11 = mul2(o11, half);
+            if (!(rh.x > 0.f)) o00.x = o01.x = o11.x = sPx.x = sPy.x = 0.f;
+            if (!(rh.y > 0.f)) o00.y = o01.y = o11.y = sPx.y = sPy.y = 0.f;
             float *ob = &sm.ob[b][warp][0][2 + v * kTexP + u + 2];
             ob[0] = o00.x; ob[kTexP] = o00.y;
             ob[kObN] = o01.x; ob[kObN + kTexP] = o01.y;
             ob[2 * kObN] = o11.x; ob[2 * kObN + kTexP] = o11.y;
             if (it > 0) {
-                float vx = fmaf(rh.x, sPx.x, rh.y * sPx.y), vy = fmaf(rh.x, sPy.x, rh.y * sPy.y);
+                float vx = sPx.x + sPx.y, vy = sPy.x + sPy.y;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     // through Omega's sampling position (half a texel per raw px)
