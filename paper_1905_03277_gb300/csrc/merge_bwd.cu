@@ -314,6 +314,9 @@ __global__ void __launch_bounds__(kBwdThreads, 4) k_merge_bwd(
                     ob1 = fmaf(t1, Pyv, ob1);
                     ob2 = fmaf(t2, Pyv, ob2);
                 }
+            // a frame rejected at the pixel is not in its channels' sums, so its weights have no bound: it
+            // is left out, where 0 times them may be no number
+            if (!(mrh < 0.f)) sPx = sPy = ob0 = ob1 = ob2 = 0.f;
             // d L / d v through the offsets d (d = q - x0 - v): -2 sum qb P; Omega-bar = -qb P P^T
             float vbx = -2.f * sPx, vby = -2.f * sPy;
             ob0 = -ob0;

@@ -20,6 +20,8 @@ CASES = [  # (scale, tile)
     ((1, 1), 32),
     ((3, 2), 16),
     ((2, 1), 16),
+    ((1, 1), 8),    # the per-pixel kernel
+    ((4, 3), 16),
 ]
 
 
