@@ -2,14 +2,27 @@
 // merge_bwd_region.cu).
 #pragma once
 
+#include <float.h>
+
 #include "hmfsr_internal.cuh"
 
 namespace hmfsr {
 namespace {
 
+// s + e plus o + oe, e and oe the rounding errors carried so far: s takes the rounded sum, e the
+// errors and that rounding's exact error (two-sum)
+__device__ __forceinline__ void two_sum(float &s, float &e, float o, float oe) {
+    const float t = s + o, bp = t - s;
+    e = (e + oe) + ((s - (t - bp)) + (o - bp));
+    s = t;
+}
+
+// the error to go with a sum: none where the sum left the range (infinity less itself is no number)
+__device__ __forceinline__ float error_of(float s, float e) { return fabsf(s) <= FLT_MAX ? e : 0.f; }
+
 // Block sums in a fixed order without FP64 arithmetic per element (FP64 is scarce on this
-// GPU): each warp adds its lanes' values by butterflies carrying the exact rounding error
-// of every FP32 addition (two-sum), lane 0 stores the warp's (sum, error) pair; the
+// GPU): each warp adds its lanes' values by butterflies carrying the exact
+// rounding error of every FP32 addition, lane 0 stores the warp's (sum, error) pair; the
 // caller's thread 0 then adds the warps' pairs in FP64 in warp order.
 template <int K>
 __device__ __forceinline__ void warp_sums_comp(float (&v)[K], float (&e)[K]) {
@@ -18,13 +31,10 @@ __device__ __forceinline__ void warp_sums_comp(float (&v)[K], float (&e)[K]) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-        for (int q = 0; q < K; ++q) {
-            const float a = v[q], b = __shfl_xor_sync(0xffffffffu, v[q], o);
-            const float t = a + b, bp = t - a;
-            const float err = (a - (t - bp)) + (b - bp);
-            e[q] = (e[q] + __shfl_xor_sync(0xffffffffu, e[q], o)) + err;
-            v[q] = t;
-        }
+        for (int q = 0; q < K; ++q)
+            two_sum(v[q], e[q], __shfl_xor_sync(0xffffffffu, v[q], o), __shfl_xor_sync(0xffffffffu, e[q], o));
+#pragma unroll
+    for (int q = 0; q < K; ++q) e[q] = error_of(v[q], e[q]);
 }
 
 // The six kernel parameters' contribution of one texel.  With k_x = s_x^2 the kernel

@@ -576,7 +576,7 @@ __global__ void __launch_bounds__(kRedThreads) k_motion_reduce(const float2 *__r
                 comp_add(sy, cy, vb.y);
             }
     }
-    double dx = (double)sx + (double)cx, dy = (double)sy + (double)cy;
+    double dx = (double)sx + (double)error_of(sx, cx), dy = (double)sy + (double)error_of(sy, cy);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         dx += __shfl_xor_sync(0xffffffffu, dx, o);

@@ -52,6 +52,10 @@ template <> struct AdjointShape<2, 1> { static constexpr int kSy = 1, kBlocks = 
 constexpr int kObN = 100;        // a phase's 8 x 8 texels, rows of 12 with zeros around
 constexpr int kObT = 14 * kTexP; // gathered along x: rows -3 .. 10 (zeros outside 0 .. 7)
 
+// Motion contributions are summed times this (exactly): a warp's 64 pixels, or an 8 x 8 block's
+// texels, cannot leave FP32's range together where each is inside it, and FP64 takes over from there
+constexpr float kPart = 1.f / 64.f;
+
 template <int S, int kSy>
 struct AdjointSmem {
     RegionSmem<S> st;
@@ -268,34 +272,25 @@ __global__ void __launch_bounds__(32 * AdjointShape<SN, SD>::kSy *RegionScale<SN
             ob[kObN] = o01.x; ob[kObN + kTexP] = o01.y;
             ob[2 * kObN] = o11.x; ob[2 * kObN + kTexP] = o11.y;
             if (it > 0) {
-                float vx = sPx.x + sPx.y, vy = sPy.x + sPy.y;
+                float vx = fmaf(kPart, sPx.x, kPart * sPx.y), vy = fmaf(kPart, sPy.x, kPart * sPy.y);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     // through Omega's sampling position (half a texel per raw px)
                     const float A0 = h ? o00.y : o00.x, A1 = h ? o01.y : o01.x, A2 = h ? o11.y : o11.x;
                     const float tr2 = A0 + A2, mA1 = -0.5f * A1;
-                    vx = fmaf(0.5f, fmaf(tr2, xa[h].x, fmaf(A2, xa[h].y, fmaf(mA1, xb[h].x, A0 * xb[h].y))), vx);
-                    vy = fmaf(0.5f, fmaf(tr2, ya[h].x, fmaf(A2, ya[h].y, fmaf(mA1, yb[h].x, A0 * yb[h].y))), vy);
+                    vx = fmaf(0.5f * kPart, fmaf(tr2, xa[h].x, fmaf(A2, xa[h].y, fmaf(mA1, xb[h].x, A0 * xb[h].y))), vx);
+                    vy = fmaf(0.5f * kPart, fmaf(tr2, ya[h].x, fmaf(A2, ya[h].y, fmaf(mA1, yb[h].x, A0 * yb[h].y))), vy);
                 }
                 // the warp's sums: lanes 0-15 take x, 16-31 y; every addition's rounding error is
                 // carried along (two-sum)
                 float a = lane < 16 ? vx : vy, ae = 0.f;
-                {
-                    const float o2 = __shfl_xor_sync(0xffffffffu, lane < 16 ? vy : vx, 16);
-                    const float q = a + o2, bp = q - a;
-                    ae = (a - (q - bp)) + (o2 - bp);
-                    a = q;
-                }
+                two_sum(a, ae, __shfl_xor_sync(0xffffffffu, lane < 16 ? vy : vx, 16), 0.f);
 #pragma unroll
-                for (int q = 8; q > 0; q >>= 1) {
-                    const float o2 = __shfl_xor_sync(0xffffffffu, a, q), oe = __shfl_xor_sync(0xffffffffu, ae, q);
-                    const float r = a + o2, bp = r - a;
-                    ae = (ae + oe) + ((a - (r - bp)) + (o2 - bp));
-                    a = r;
-                }
+                for (int q = 8; q > 0; q >>= 1)
+                    two_sum(a, ae, __shfl_xor_sync(0xffffffffu, a, q), __shfl_xor_sync(0xffffffffu, ae, q));
                 if ((lane & 15) == 0)
                     vbar_region[(((((size_t)f * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * gridDim.z + blockIdx.z) * NW + warp) * 2 + (lane >> 4)] =
-                        make_float2(a, ae);
+                        make_float2(a, error_of(a, ae));
                 float *plane = rhbar_phase + ((size_t)f * (S * S) + (size_t)(sy * S + sx)) * ((size_t)hg * wg);
                 if (in0) plane[rp] = rhb.x;
                 if (in1) plane[rp + wg] = rhb.y;
@@ -480,7 +475,7 @@ __global__ void __launch_bounds__(kRpW *kRpH) k_rpath_region(const float *__rest
             }
         if (__float_as_int(s_rh[ty + 2][tx + 2].y) & 0x80) {  // R unclamped
             const float4 d = rb[(size_t)f * hw + (size_t)v * g.wh + u];
-            vb = make_float2(rbar * d.y, rbar * d.z);
+            vb = make_float2(kPart * (rbar * d.y), kPart * (rbar * d.z));
             pv[0] = rbar * d.w;
             pv[1] = -rbar;
         }
@@ -552,7 +547,8 @@ __global__ void __launch_bounds__(128) k_motion_region(const float2 *__restrict_
         x += __shfl_xor_sync(0xffffffffu, x, o);
         y += __shfl_xor_sync(0xffffffffu, y, o);
     }
-    if (l == 0 && t < g.n * ntl) grad_motion[t] = make_float2((float)x, (float)y);
+    constexpr double kWhole = 1.0 / kPart;
+    if (l == 0 && t < g.n * ntl) grad_motion[t] = make_float2((float)(kWhole * x), (float)(kWhole * y));
 }
 
 template <int SN, int SD>
