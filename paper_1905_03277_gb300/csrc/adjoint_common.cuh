@@ -21,15 +21,15 @@ __device__ __forceinline__ void two_sum(float &s, float &e, float o, float oe) {
 __device__ __forceinline__ float error_of(float s, float e) { return fabsf(s) <= FLT_MAX ? e : 0.f; }
 
 // Block sums in a fixed order without FP64 arithmetic per element (FP64 is scarce on this
-// GPU): each warp adds its lanes' values by butterflies carrying the exact
+// GPU): each warp (or group of kLanes) adds its lanes' values by butterflies carrying the exact
 // rounding error of every FP32 addition, lane 0 stores the warp's (sum, error) pair; the
 // caller's thread 0 then adds the warps' pairs in FP64 in warp order.
-template <int K>
+template <int K, int kLanes = 32>
 __device__ __forceinline__ void warp_sums_comp(float (&v)[K], float (&e)[K]) {
 #pragma unroll
     for (int q = 0; q < K; ++q) e[q] = 0.f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
+    for (int o = kLanes / 2; o > 0; o >>= 1)
 #pragma unroll
         for (int q = 0; q < K; ++q)
             two_sum(v[q], e[q], __shfl_xor_sync(0xffffffffu, v[q], o), __shfl_xor_sync(0xffffffffu, e[q], o));

@@ -260,7 +260,7 @@ struct BwdPlanes {
     // the region kernels (merge_bwd_region.cu) instead of the *_pix, *_rows and *_tex planes above:
     float *rhbar_phase;     // [n][S*S phases][half-res grid] dL/dRhat at output pixels, by phase
     float2 *vbar_region;    // [n][regions][phases]{x, y} motion contributions through the weights, with rounding errors
-    float2 *vbar_block;     // [n][8 x 8-texel blocks] motion contributions through R
+    float4 *vbar_block;     // [n][8 x 8-texel blocks] motion contributions through R, {x, its rounding error, y, its}
     int n_bwd_blocks, n_rp_blocks;
 };
 size_t carve_backward(void *ws, const Geom &g, int snum, int sden, size_t fwd_bytes, BwdPlanes *B);

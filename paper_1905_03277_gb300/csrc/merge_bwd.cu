@@ -632,7 +632,7 @@ size_t carve_backward(void *ws, const Geom &g, int snum, int sden, size_t fwd_by
         const BwdRegionSizes z = bwd_region_sizes(g, snum, sden);
         B->rhbar_phase = (float *)take(sizeof(float) * z.rhbar);
         B->vbar_region = (float2 *)take(sizeof(float2) * z.vregion);
-        B->vbar_block = (float2 *)take(sizeof(float2) * z.vblock);
+        B->vbar_block = (float4 *)take(sizeof(float4) * z.vblock);
         B->n_bwd_blocks = z.bwd_blocks;
         B->n_rp_blocks = z.rp_blocks;
         B->part6 = (double *)take(sizeof(double) * 6 * (size_t)B->n_bwd_blocks);

@@ -272,19 +272,25 @@ __global__ void __launch_bounds__(32 * AdjointShape<SN, SD>::kSy *RegionScale<SN
             ob[kObN] = o01.x; ob[kObN + kTexP] = o01.y;
             ob[2 * kObN] = o11.x; ob[2 * kObN + kTexP] = o11.y;
             if (it > 0) {
-                float vx = fmaf(kPart, sPx.x, kPart * sPx.y), vy = fmaf(kPart, sPy.x, kPart * sPy.y);
+                const float2 part = make_float2(kPart, kPart);
+                float2 vx = mul2(sPx, part), vy = mul2(sPy, part);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     // through Omega's sampling position (half a texel per raw px)
                     const float A0 = h ? o00.y : o00.x, A1 = h ? o01.y : o01.x, A2 = h ? o11.y : o11.x;
                     const float tr2 = A0 + A2, mA1 = -0.5f * A1;
-                    vx = fmaf(0.5f * kPart, fmaf(tr2, xa[h].x, fmaf(A2, xa[h].y, fmaf(mA1, xb[h].x, A0 * xb[h].y))), vx);
-                    vy = fmaf(0.5f * kPart, fmaf(tr2, ya[h].x, fmaf(A2, ya[h].y, fmaf(mA1, yb[h].x, A0 * yb[h].y))), vy);
+                    const float px = fmaf(tr2, xa[h].x, fmaf(A2, xa[h].y, fmaf(mA1, xb[h].x, A0 * xb[h].y)));
+                    const float py = fmaf(tr2, ya[h].x, fmaf(A2, ya[h].y, fmaf(mA1, yb[h].x, A0 * yb[h].y)));
+                    if (h) { vx.y = fmaf(0.5f * kPart, px, vx.y); vy.y = fmaf(0.5f * kPart, py, vy.y); }
+                    else { vx.x = fmaf(0.5f * kPart, px, vx.x); vy.x = fmaf(0.5f * kPart, py, vy.x); }
                 }
                 // the warp's sums: lanes 0-15 take x, 16-31 y; every addition's rounding error is
-                // carried along (two-sum)
-                float a = lane < 16 ? vx : vy, ae = 0.f;
-                two_sum(a, ae, __shfl_xor_sync(0xffffffffu, lane < 16 ? vy : vx, 16), 0.f);
+                // carried along (two-sum), from the lane's two pixels on
+                const bool lo = lane < 16;
+                float a = lo ? vx.x : vy.x, ae = 0.f, o2 = lo ? vy.x : vx.x, oe = 0.f;
+                two_sum(a, ae, lo ? vx.y : vy.y, 0.f);
+                two_sum(o2, oe, lo ? vy.y : vx.y, 0.f);
+                two_sum(a, ae, __shfl_xor_sync(0xffffffffu, o2, 16), __shfl_xor_sync(0xffffffffu, oe, 16));
 #pragma unroll
                 for (int q = 8; q > 0; q >>= 1)
                     two_sum(a, ae, __shfl_xor_sync(0xffffffffu, a, q), __shfl_xor_sync(0xffffffffu, ae, q));
@@ -385,13 +391,13 @@ template <int SN, int SD>
 __global__ void __launch_bounds__(kRpW *kRpH) k_rpath_region(const float *__restrict__ rhbar_phase,
                                                              const unsigned char *__restrict__ flags,
                                                              const float4 *__restrict__ rb, Geom g,
-                                                             float2 *__restrict__ vbar_block,
+                                                             float4 *__restrict__ vbar_block,
                                                              double *__restrict__ partials) {
     constexpr int S = RegionScale<SN, SD>::S, kOff = RegionScale<SN, SD>::kOff;
     __shared__ float s_x[S][kRpHaloH + 1][kRpHaloW];
     __shared__ float2 s_rh[kRpHaloH][kRpHaloW];  // Rhat-bar, and the code of the offset its window picked
     __shared__ double s_red[kRpH][4];
-    __shared__ float2 s_vb[kRpH][4];
+    __shared__ float4 s_vb[kRpH][4];  // {x, its error, y, its error}
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, f = blockIdx.z;
     const int u0 = blockIdx.x * kRpW, v0 = blockIdx.y * kRpH;
     const size_t hw = (size_t)g.hh * g.wh;
@@ -460,8 +466,7 @@ __global__ void __launch_bounds__(kRpW *kRpH) k_rpath_region(const float *__rest
     }
     __syncthreads();
     const int u = u0 + tx, v = v0 + ty;
-    float pv[2] = {0.f, 0.f}, pe[2];
-    float2 vb = make_float2(0.f, 0.f);
+    float pv[2] = {0.f, 0.f}, pe[2], vb[2] = {0.f, 0.f}, ve[2];
     if (u < g.wh && v < g.hh) {
         // R-bar(u, v): the windows centred at (u + i, v + j) that picked offset (-i, -j)
         float rbar = 0.f;
@@ -475,61 +480,64 @@ __global__ void __launch_bounds__(kRpW *kRpH) k_rpath_region(const float *__rest
             }
         if (__float_as_int(s_rh[ty + 2][tx + 2].y) & 0x80) {  // R unclamped
             const float4 d = rb[(size_t)f * hw + (size_t)v * g.wh + u];
-            vb = make_float2(kPart * (rbar * d.y), kPart * (rbar * d.z));
+            vb[0] = kPart * (rbar * d.y);
+            vb[1] = kPart * (rbar * d.z);
             pv[0] = rbar * d.w;
             pv[1] = -rbar;
         }
     }
     // 8 x 8-texel sums of the motion contributions
-#pragma unroll
-    for (int q = 4; q > 0; q >>= 1) {
-        vb.x += __shfl_xor_sync(0xffffffffu, vb.x, q);
-        vb.y += __shfl_xor_sync(0xffffffffu, vb.y, q);
-    }
-    if ((tx & 7) == 0) s_vb[ty][tx >> 3] = vb;
+    warp_sums_comp<2, 8>(vb, ve);
+    if ((tx & 7) == 0) s_vb[ty][tx >> 3] = make_float4(vb[0], ve[0], vb[1], ve[1]);
     warp_sums_comp<2>(pv, pe);
     if (tx == 0) {
         s_red[ty][0] = (double)pv[0]; s_red[ty][1] = (double)pe[0];
         s_red[ty][2] = (double)pv[1]; s_red[ty][3] = (double)pe[1];
     }
     __syncthreads();
-    if (threadIdx.x < 4 * (kRpH / 8)) {
-        const int bx = blockIdx.x * 4 + (threadIdx.x & 3), by = blockIdx.y * (kRpH / 8) + (threadIdx.x >> 2);
-        const int nbx = div_up(g.wh, 8), nby = div_up(g.hh, 8);
-        double x = 0.0, y = 0.0;
-        for (int r = 0; r < 8; ++r) {
-            const float2 q = s_vb[(threadIdx.x >> 2) * 8 + r][threadIdx.x & 3];
-            x += (double)q.x;
-            y += (double)q.y;
+    if (threadIdx.x < 4 * kRpH) {  // a lane's row of a block: four blocks' rows in a warp
+        const int k = threadIdx.x & 3, r = threadIdx.x >> 2;
+        const float4 q = s_vb[r][k];
+        float x = q.x, xe = q.y, y = q.z, ye = q.w;
+#pragma unroll
+        for (int o = 4; o < 32; o *= 2) {
+            two_sum(x, xe, __shfl_xor_sync(0xffffffffu, x, o), __shfl_xor_sync(0xffffffffu, xe, o));
+            two_sum(y, ye, __shfl_xor_sync(0xffffffffu, y, o), __shfl_xor_sync(0xffffffffu, ye, o));
         }
-        if (bx < nbx && by < nby) vbar_block[((size_t)f * nby + by) * nbx + bx] = make_float2((float)x, (float)y);
-    } else if (threadIdx.x >= 32 && threadIdx.x < 34) {
-        const int q = threadIdx.x - 32;
+        const int bx = blockIdx.x * 4 + k, by = blockIdx.y * (kRpH / 8) + (r >> 3);
+        const int nbx = div_up(g.wh, 8), nby = div_up(g.hh, 8);
+        if ((r & 7) == 0 && bx < nbx && by < nby)
+            vbar_block[((size_t)f * nby + by) * nbx + bx] = make_float4(x, error_of(x, xe), y, error_of(y, ye));
+    } else if (threadIdx.x < 4 * kRpH + 2) {
+        const int q = threadIdx.x - 4 * kRpH;
         double acc = 0.0;
         for (int r = 0; r < kRpH; ++r) acc += s_red[r][2 * q] + s_red[r][2 * q + 1];
         partials[bid * 2 + q] = acc;
     }
 }
 
-// Every tile's motion gradient: its regions' and its 8 x 8-texel blocks' sums, in a fixed order.
-// Eight lanes per tile, so that a tile's loads (up to 16 parts of each region) are in flight
-// together: latency is all of it.  One lane per tile took 23 us for the 256 x 320 x 4 crop at 2x
-// and 17 for 1 MP x 8 at 3/2; this 8 and 18 (FP64 sums:
-// FP32 with the rounding errors carried took 9, but makes an infinite sum a NaN).
+// Every tile's motion gradient: its regions' and its 8 x 8-texel blocks' sums, in a fixed order, in
+// FP64; their rounding errors, 2^-24 of them and less, in FP32 beside it.  Eight lanes per tile, so
+// that a tile's loads (up to 16 parts of each region) are in flight together: latency and the FP64
+// additions are all of it.  1 MP x 8 at 3/2: 16 us (20 with the errors in FP64 too); the
+// 256 x 320 x 4 crop at 2x: 7 us (23 with one lane per tile).
 constexpr int kTileLanes = 8;
-__global__ void __launch_bounds__(128) k_motion_region(const float2 *__restrict__ vbar_region, const float2 *__restrict__ vbar_block,
+__global__ void __launch_bounds__(128) k_motion_region(const float2 *__restrict__ vbar_region, const float4 *__restrict__ vbar_block,
                                                        Geom g, int off, int parts, float2 *__restrict__ grad_motion) {
     const int t = (blockIdx.x * 128 + threadIdx.x) / kTileLanes, l = threadIdx.x % kTileLanes;
     const int ntl = g.ty * g.tx, f = t / ntl, r = t - f * ntl, ty = r / g.tx, tx = r - ty * g.tx;
     double x = 0.0, y = 0.0;
+    float xe = 0.f, ye = 0.f;
     if (t < g.n * ntl && f != g.ref) {
         const int nb = g.tile / 16, nbx = div_up(g.wh, 8), nby = div_up(g.hh, 8);
         const int x0 = tx * nb, y0 = ty * nb, bw = min(x0 + nb, nbx) - x0, bh = min(y0 + nb, nby) - y0;
         for (int k = l; k < bw * bh; k += kTileLanes) {
             const int by = k / bw, bx = k - by * bw;
-            const float2 q = __ldg(vbar_block + ((size_t)f * nby + y0 + by) * nbx + x0 + bx);
+            const float4 q = __ldg(vbar_block + ((size_t)f * nby + y0 + by) * nbx + x0 + bx);
             x += (double)q.x;
-            y += (double)q.y;
+            y += (double)q.z;
+            xe += q.y;
+            ye += q.w;
         }
         // regions are the same 8 x 8 texels, after `off` leading ones that belong to the first tiles
         const int nrx = nbx + off, nry = nby + off;
@@ -538,10 +546,14 @@ __global__ void __launch_bounds__(128) k_motion_region(const float2 *__restrict_
             const int q0 = k / parts, by = q0 / rw, bx = q0 - by * rw;
             const float4 q = __ldg(reinterpret_cast<const float4 *>(vbar_region) +
                                    (((size_t)f * nry + ry0 + by) * nrx + rx0 + bx) * parts + (k - q0 * parts));
-            x += (double)q.x + (double)q.y;
-            y += (double)q.z + (double)q.w;
+            x += (double)q.x;
+            y += (double)q.z;
+            xe += q.y;
+            ye += q.w;
         }
     }
+    x += (double)xe;
+    y += (double)ye;
 #pragma unroll
     for (int o = kTileLanes / 2; o > 0; o >>= 1) {
         x += __shfl_xor_sync(0xffffffffu, x, o);
