@@ -567,9 +567,12 @@ hmfsr_status hmfsr_batch_run(hmfsr_batch_plan plan, const uint16_t *const *burst
     if (!plan || !bursts_dev || !rgb_dev) return HMFSR_ERR_INVALID_ARG;
     if (!ws || ws_bytes < plan->ws_bytes || (reinterpret_cast<uintptr_t>(ws) & 255)) return HMFSR_ERR_WORKSPACE;
     char *base = static_cast<char *>(ws);
+    for (int b = 0; b < plan->nb; ++b)  // a refused call leaves the plan as it was
+        if (!bursts_dev[b] || !rgb_dev[b] || (reinterpret_cast<uintptr_t>(bursts_dev[b]) & 3) ||
+            (motion_dev && (reinterpret_cast<uintptr_t>(motion_dev[b]) & 7)))
+            return HMFSR_ERR_INVALID_ARG;
     bool moved = false;  // some pointer is not the last call's
     for (int b = 0; b < plan->nb; ++b) {
-        if (!bursts_dev[b] || !rgb_dev[b] || (reinterpret_cast<uintptr_t>(bursts_dev[b]) & 3)) return HMFSR_ERR_INVALID_ARG;
         BatchBurst &bb = plan->host[b];
         const float *old_motion = bb.motion;
         moved = moved || bb.burst != bursts_dev[b] || bb.rgb != rgb_dev[b];
@@ -592,7 +595,6 @@ hmfsr_status hmfsr_batch_run(hmfsr_batch_plan plan, const uint16_t *const *burst
         bb.P.geo = reinterpret_cast<int4 *>(base + off); off = align256(off + sizeof(int4) * (size_t)g.n * g.ty * g.tx);
         float *own_motion = reinterpret_cast<float *>(base + off);
         bb.motion = (motion_dev && motion_dev[b]) ? motion_dev[b] : own_motion;
-        if (reinterpret_cast<uintptr_t>(bb.motion) & 7) return HMFSR_ERR_INVALID_ARG;
         moved = moved || bb.motion != old_motion;
     }
     if (moved) plan->tables_valid = plan->graph_current = false;

@@ -1,5 +1,5 @@
 """A batch plan run on other buffers than before (hmfsr_batch_run): every mode reads the bursts and
-writes the outputs and motions of this call."""
+writes the outputs and motions of this call, also where a refused call came in between."""
 import pytest
 import torch
 
@@ -58,3 +58,18 @@ def test_second_buffers(two, mode):
     m3 = [m2[0], torch.full_like(m2[1], 7.0), m2[2]]
     plan.run(bursts2, o2, m3, wait=True)
     check(o2 + m3, rgbs2 + mvs2)
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+def test_refused_call_between(two, mode):
+    dev, ((bursts, mvs, rgbs), (bursts2, _, rgbs2)) = two
+    plan = hm.BatchPlan(SHAPES, hm.MergeParams(noise_a=1.0, noise_b=9.0))
+    plan.set_mode(mode)
+    o, m = buffers(plan, dev)
+    for _ in range(2):
+        plan.run(bursts, o, m, wait=True)
+    odd = torch.zeros(bursts[1].numel() + 1, dtype=bursts[1].dtype, device=dev)[1:].view(bursts[1].shape)
+    with pytest.raises(RuntimeError, match="invalid argument"):  # 2-byte aligned
+        plan.run([bursts2[0], odd, bursts[2]], o, m)
+    plan.run([bursts2[0], bursts[1], bursts[2]], o, m, wait=True)
+    check(o, [rgbs2[0], rgbs[1], rgbs[2]])
