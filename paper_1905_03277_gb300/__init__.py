@@ -736,8 +736,9 @@ class BatchPlan:
         _lib.check(st, "batch")
         return st
 
-    def configure(self, merge_tile_w: int = 32, ctas_per_sm: int = 0, regs_variant: int = 1, queue_order: int = 0,
+    def configure(self, merge_tile_w: int = 32, ctas_per_sm: int = 0, regs_variant: int = 0, queue_order: int = 0,
                   spin_limit: int = 1 << 22, inject_stall: bool = False):
+        """hmfsr_batch_configure; what is left out is what a new plan has."""
         _lib.check(self._L.hmfsr_batch_configure(self._h, merge_tile_w, ctas_per_sm, regs_variant, queue_order,
                                                  spin_limit, int(inject_stall)), "hmfsr_batch_configure")
 
