@@ -492,7 +492,6 @@ hmfsr_status hmfsr_batch_plan_create(const hmfsr_burst_desc *descs, int n_bursts
     p->prof_off = off; off = align256(off + 3 * S_COUNT * sizeof(unsigned long long));
     for (int b = 0; b < n_bursts; ++b) {
         BatchBurst &bb = p->host[b];
-        memset(&bb, 0, sizeof(bb));
         const hmfsr_burst_desc &d = descs[b];
         Geom &g = bb.g;
         g.n = d.n_frames; g.h = d.height; g.w = d.width; g.pitch = d.pitch_elems; g.ref = d.ref; g.wl = d.white_level;
