@@ -101,12 +101,6 @@ __device__ __forceinline__ void copy4(float *dst, const float *src) {
 }
 __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// n / d from the SFU reciprocal with one residual correction
-__device__ __forceinline__ float ratio(float n, float d) {
-    const float r = fast_rcp(d), q = n * r;
-    return fmaf(fmaf(-q, d, n), r, q);
-}
-
 // keeps a value that a loop uses in its register: without it the compiler derives it again
 // (index divisions, clamps) in every iteration to save the register
 __device__ __forceinline__ void keep(int &x) { asm volatile("" : "+r"(x)); }
@@ -654,9 +648,9 @@ __device__ __forceinline__ void merge_region(RegionSmem<RegionScale<SN, SD>::S> 
                     continue;
                 }
             }
-            HMFSR_ST(rgb + o, ratio(p.numR, p.denR));
-            HMFSR_ST(rgb + po + o, ratio(p.numG, p.denG));
-            HMFSR_ST(rgb + 2 * po + o, ratio(p.numB, p.denB));
+            HMFSR_ST(rgb + o, p.numR / p.denR);
+            HMFSR_ST(rgb + po + o, p.numG / p.denG);
+            HMFSR_ST(rgb + 2 * po + o, p.numB / p.denB);
             if (kDen) {
                 HMFSR_ST(den_out + o, log2f(p.denR) - p.mR);
                 HMFSR_ST(den_out + po + o, log2f(p.denG) - p.mG);
