@@ -405,7 +405,7 @@ def run_gpu(args):
         torch.cuda.synchronize()
         tuning[fn] = t0.elapsed_time(t1) / 5
     tuning["noise_table"] = (f"{ntab.shape[0]} levels x 4096 trials x 54 Philox-4x32-10 Irwin-Hall normals "
-                             "(FP64 samples, rounding and clipping)")
+                             "(samples rounded and clipped as in FP64)")
 
     # bounded memory: the same merge a chunk of frames at a time (the running sums of every
     # output pixel kept in the workspace between chunks), against the resident merge

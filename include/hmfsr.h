@@ -256,8 +256,10 @@ size_t hmfsr_batch_workspace_size(hmfsr_batch_plan plan);
 /* Run the batch on `stream`: bursts_dev[b] (uint16, layout of desc b), rgb_dev[b]
  * (float32 [3][Ho][Wo], written) and optionally motion_dev[b] (float32 [n][TY][TX][2],
  * written; NULL array or entries: kept in the workspace).  Host arrays of device
- * pointers.  The first run, or a run with a different workspace, stream or grid,
- * captures and instantiates the CUDA graph; later runs replay it.  The call returns
+ * pointers; a call that refuses one leaves the plan as it was.  The first run, or a run
+ * with a different workspace, stream or grid, captures and instantiates the CUDA graph;
+ * later runs replay it.  Other pointers than the last run's are uploaded (persistent
+ * kernel) or captured and put into the graph (per-burst kernels).  The call returns
  * after enqueueing; hmfsr_batch_wait reports the outcome. */
 hmfsr_status hmfsr_batch_run(hmfsr_batch_plan plan, const uint16_t *const *bursts_dev, float *const *motion_dev,
                              float *const *rgb_dev, void *ws, size_t ws_bytes, void *stream);

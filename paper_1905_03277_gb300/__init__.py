@@ -487,8 +487,7 @@ def merge_prepare(burst: torch.Tensor, motion: torch.Tensor, params: MergeParams
     stream = _on(burst.device, stream)
     nbytes = L.hmfsr_workspace_size(_lib.OP_MERGE_STAGES, ctypes.byref(d), params.tile, 1, 1)
     if workspace is None:
-        s = stream if stream is not None else torch.cuda.current_stream(burst.device)
-        with torch.cuda.stream(s):
+        with torch.cuda.stream(stream):
             buf = torch.empty(nbytes + 256, dtype=torch.uint8, device=burst.device)
         off = (-buf.data_ptr()) % 256
         ws = buf[off:off + nbytes]

@@ -12,11 +12,12 @@
 // in shared memory a frame ahead, and the squared cross products of det(Omega) (omega_form) are
 // formed once per texel cell instead of once per pixel.
 //
-// What bounds it: issue and shared-memory bandwidth, 12 MP x 8 at scale 1: ~225 warp-instructions
-// per 32 pixel-frames (the 2 x 2-pixel kernel it replaces: 271), issue 60 %, shared-memory data
-// path 80 %; DRAM 10 %.  One box, accumulation call:
-//   12 MP x 8, 1x    1147 -> 916 us      12 MP x 8, 1.5x   2756 -> 1947 us
-//   12 MP x 15, 2x   8568 -> 5320 us     0.07 MP x 8, 1x     57 -> 38 us
+// What bounds it: issue and shared-memory bandwidth, 12 MP x 8 at scale 1: 244 warp-instructions
+// per 32 pixel-frames (the 2 x 2-pixel kernel it replaces: 271), issue 68 %, shared-memory data
+// path 77 %; DRAM 0.9 TB/s; 882 us (ncu).  Calls of hmfsr_merge_accumulate (CUDA events), with the
+// per-pixel kernels and now:
+//   12 MP x 8, 1x    1147 -> 908 us      12 MP x 8, 1.5x   2756 -> 1964 us
+//   12 MP x 15, 2x   8568 -> 5342 us     0.07 MP x 8, 1x     57 -> 33 us
 #pragma once
 
 #include <limits.h>
@@ -245,8 +246,8 @@ struct RegionStage {
     }
     // pairs of raw samples, as they are, into registers or the even plane; spread_raw turns a thread's
     // own pairs into the two planes once they have arrived.  Registers cost less at the shared-memory
-    // path (merging at scale 1, which that path bounds: 916 us against 931 at 12 MP x 8), shared
-    // memory where registers are short (3/2: 1947 us against 1960; the adjoint, which spilled).
+    // path (merging at scale 1, which that path bounds: 1.6 % of the call at 12 MP x 8), shared
+    // memory where registers are short (3/2: 0.7 %; the adjoint, which spilled).
     __device__ __forceinline__ void stage_raw(float *dst, int it) {
         const typename Smem::Desc &d = desc(it);
         const uint16_t *p = d.raw;

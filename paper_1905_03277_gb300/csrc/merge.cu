@@ -112,10 +112,11 @@ __global__ void __launch_bounds__(128, (NY == 2 ? 4 : 5)) k_merge_q1_chunk(const
                                        blockIdx.x * stage::kQuadW + 2 * qx, blockIdx.y * 8 * NY + NY * qy, io);
 }
 
-// A region's output pixels (stage::merge_region): threads and blocks per SM by scale.  Measured
-// on the 12-MP bursts (accumulation call): 1x, 128 threads: 5 blocks per SM 930 us, 6 (spills)
-// 965, 4 1006; 1.5x, 288 threads: 3 blocks 1921 us, 2 2125; 2x, 256 threads, two x phases each:
-// 2 blocks 5315 us (128 threads x 4 5605; one phase each, 256 x 3, 6076).
+// A region's output pixels (stage::merge_region): threads and blocks per SM by scale.  The others
+// tried on the 12-MP bursts, as the accumulation call's time over that of the one taken: 1x, 128
+// threads and 5 blocks per SM (6 blocks, which spill, 1.04; 4 blocks 1.08); 1.5x, 288 threads, 3
+// blocks (2 blocks 1.11); 2x, 256 threads with two x phases each, 2 blocks (128 threads, 4 blocks
+// 1.05; one phase each, 256 threads, 3 blocks 1.14).
 template <int SN, int SD>
 struct RegionShape;
 template <> struct RegionShape<1, 1> { static constexpr int kThreads = 128, kBlocks = 5, kNpx = 1; };

@@ -14,9 +14,9 @@
 //     gather onto texels has constant weights.
 // Fixed orders everywhere, so results are deterministic.
 //
-// Bounded by the issue rate (57 %) with the shared-memory path at 56 %: 645 warp-instructions per
-// 32 pixel-frames.  At 1 MP x 8 frames, scale 3/2 (the fitting workload) the main kernel takes 540 us
-// where the per-pixel one takes 802, the R-hat path 68 where its two kernels take 106.  Registers
+// Bounded by the issue rate (57 %) with the shared-memory path at 60 %: 659 warp-instructions per
+// 32 pixel-frames.  At 1 MP x 8 frames, scale 3/2 (the fitting workload) the main kernel takes 550 us
+// where the per-pixel one takes 802, the R-hat path 70 where its two kernels take 106.  Registers
 // decide the rest: shared memory leaves little L1, so every word spilled in the frame loop goes to
 // L2 (a version with 16 spilled words took 654 us).  Hence staging through shared memory and not
 // registers, small blocks of one row of phases (3 warps, 5 blocks per SM; all nine phases in one

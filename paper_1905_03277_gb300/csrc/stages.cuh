@@ -1210,7 +1210,7 @@ __device__ __forceinline__ void hf_flag_px(const uint16_t *__restrict__ burst, c
 // 158); packed pairs with a row fetched ahead take 110 registers and more time than they save (150
 // to 190 us), and frames side by side in a block, sharing the base row, 230.  The guide sums stay
 // as the mantissa of 2^23 (exact, and so are the differences of two of them).  At 12 MP x 8 frames
-// 147 us became 138, at 256 x 256 x 8 16 us became 10.
+// 147 us became 138, at 256 x 256 x 8 16 us became 8.
 // --------------------------------------------------------------------------------------
 constexpr int kRobStrip = 64;  // default strip height, as for kPrepStrip
 constexpr float kLog2e = 1.44269504088896340736f;
