@@ -146,8 +146,12 @@ __global__ void k_rback(const uint2 *__restrict__ s1, const float4 *__restrict__
     flags[o] = unclamped ? 0x80 : 0;
 }
 
-// first minimum of R over the 5x5 window of valid pixels (scan order), offset 0..24
-__global__ void k_argmin(const float4 *__restrict__ rb, Geom g, unsigned char *__restrict__ flags) {
+// First minimum of R over the 5x5 window of valid pixels (scan order), offset 0..24; 31 (none) where
+// the forward's Rhat is 0.  R here comes from expf, the forward's from the SFU: at the boundary it can
+// be a last place above 0 where the forward rejects, and dL/dRhat of a pixel that a frame is rejected
+// at has no bound.
+__global__ void k_argmin(const float4 *__restrict__ rb, const float *__restrict__ rhat, Geom g,
+                         unsigned char *__restrict__ flags) {
     const int u = blockIdx.x * blockDim.x + threadIdx.x, v = blockIdx.y, f = blockIdx.z;
     if (u >= g.wh || f == g.ref) return;
     const size_t hw = (size_t)g.hh * g.wh;
@@ -162,6 +166,7 @@ __global__ void k_argmin(const float4 *__restrict__ rb, Geom g, unsigned char *_
             if (r < best) { best = r; bi = (j + 2) * 5 + (i + 2); }
         }
     const size_t o = (size_t)f * hw + (size_t)v * g.wh + u;
+    if (!(rhat[o] > 0.f)) bi = 31;
     flags[o] = (unsigned char)((flags[o] & 0x80) | bi);
 }
 
@@ -481,7 +486,8 @@ __global__ void __launch_bounds__(kRpThreads) k_rpath(const float *__restrict__ 
                 if (uu < 0 || uu >= g.wh || vv < 0 || vv >= g.hh) continue;
                 const size_t o = (size_t)f * hw + (size_t)vv * g.wh + uu;
                 const int bi = flags[o] & 0x1f;
-                // window of (uu,vv) picked offset bi = (dj+2)*5 + (di+2): the pixel (uu+di, vv+dj)
+                // window of (uu,vv) picked offset bi = (dj+2)*5 + (di+2): the pixel (uu+di, vv+dj); 31 is no
+                // pixel's offset (it would lie 4 rows down)
                 if (uu + (bi % 5 - 2) == u && vv + (bi / 5 - 2) == v) rbar += rhbar_tex[o];
             }
         const size_t o = (size_t)f * hw + (size_t)v * g.wh + u;
@@ -668,7 +674,7 @@ cudaError_t launch_bwd_robust(const float *motion, const Geom &g, const MergeCon
     const dim3 tex_grid(div_up(g.wh, 128), g.hh, g.n);
     k_sel<<<div_up(g.n * g.ty * g.tx, 128), 128, 0, s>>>(mv, g.n, g.ty, g.tx, c.m_th, B.sel);
     k_rback<<<tex_grid, 128, 0, s>>>(P.s1, P.base_stats, mv, P.s_tile, B.sel, g, c, B.rb, B.flags);
-    k_argmin<<<tex_grid, 128, 0, s>>>(B.rb, g, B.flags);
+    k_argmin<<<tex_grid, 128, 0, s>>>(B.rb, P.rhat, g, B.flags);
     return cudaGetLastError();
 }
 
